@@ -1,0 +1,473 @@
+#pragma once
+// KS: summation with the permuted block on chip, for layouts whose d permuted
+// indices form one dense block of O^d elements per spectator position (a
+// torch-contiguous tensor: permuted indices fastest, spectators outside, at
+// any strides).
+//
+// There the members of an orbit are scattered inside a block of O^d elements
+// (14 KB for O = 12, d = 3), so a CTA copies the blocks of NS spectator
+// positions into shared memory with unit-stride asynchronous copies, runs
+// every element orbit in shared memory and stores the blocks back with
+// unit-stride stores: each element crosses HBM once each way. The general
+// kernel KG reads and writes the same elements as scattered 8-byte accesses,
+// unranks a tuple per thread and sums with FP64 instructions: 2480 us on
+// A[32^3, 12^3], factorized Table II row 1 (0.37 TB/s), against 507 us here.
+//
+// - Canonical tuples come from a table in shared memory, grouped by equality
+//   pattern and built once per CTA, so warps run one pattern's code and no
+//   thread searches for its tuple.
+// - For even O every row, plane and volume of the block is followed by one
+//   unused element: all index strides in shared memory are odd, so lanes that
+//   step along any permuted index fall on different banks.
+// - KG's FP64 arithmetic is native FP64 in the reference order; GB300's FP64
+//   pipe (2 operations per SM per clock) limits that to 57 G elements/s on the
+//   three-factor-term chains. Here the sums run in 64-bit integers on a grid
+//   fine enough that the result is more accurate than the FP64 sum (fixed_sum
+//   below); groups outside its range, and SPINSUM_STRICT, take the FP64 order.
+#include "ss_devcache.h"
+#include "ss_k2.cuh"
+
+namespace ss {
+
+constexpr int AR_FIXED = 4;  // kernel-template choice of this file: FP64 through fixed_sum
+
+struct KsArgs {
+  int ns;             // spectator positions per round
+  int T, Tp;          // elements of a permuted block, and with its padding
+  unsigned mT, mO;    // ceil(2^32 / T), ceil(2^32 / O)
+  unsigned mO2, mO3;  // ceil(2^32 / O^2), ceil(2^32 / O^3)
+  int pad;            // 1: padded rows, planes, volumes (even O)
+  int pst[4];         // shared-memory stride of permuted index k
+  int ntot;           // canonical tuples
+  int nspectab;       // offset of the spectator-offset table in shared memory (bytes)
+  int bits;           // AR_FIXED: an input's magnitude stays below 2^bits
+  int sh0;            // AR_FIXED: result exponent offset (see fixed_sum)
+  unsigned emin, emax;
+};
+
+// quotient by a constant with its precomputed reciprocal (numerators below 2^16)
+__device__ __forceinline__ int ks_div(int n, unsigned m) { return (int)__umulhi((unsigned)n, m); }
+
+// A fixed-point value lo + hi 2^32 with a SIGNED low word, so that a product
+// with a 32-bit coefficient is one 32 x 32 -> 64-bit multiply-add and one
+// 32-bit one.
+struct Fix64 {
+  int lo, hi;
+};
+__device__ __forceinline__ Fix64 fix64(long long X) {
+  const int lo = (int)(unsigned)X;
+  return Fix64{lo, (int)(X >> 32) + (int)((unsigned)lo >> 31)};
+}
+__device__ __forceinline__ void fix64_mac(long long& acc, int c, const Fix64& x) {
+  acc += (long long)c * (long long)x.lo;
+  acc += (long long)((unsigned long long)(unsigned)(c * x.hi) << 32);
+}
+
+// FP64 value of Y * 2^sh, rounded once to nearest: the two 32-bit halves as
+// FP64 numbers with offsets 2^84 and 2^52 (times 2^sh); their difference to
+// the joint offset is exact and the last addition rounds.
+__device__ __forceinline__ double fixed_rn(long long Y, int sh) {
+  const int s = (int)((unsigned)sh << 20);
+  const double h = __hiloint2double(0x45300000 + s, (int)((unsigned)(Y >> 32) ^ 0x80000000u));
+  const double c = __hiloint2double(0x45300000 + s, (int)0x80100000u);  // 2^84 + 2^63 + 2^52
+  const double l = __hiloint2double(0x43300000 + s, (int)(unsigned)Y);
+  return __dadd_rn(__dsub_rn(h, c), l);
+}
+
+// The orbit operator of pattern P in 64-bit integers. Inputs are rounded to
+// the grid 2^(E + 1 - bits) (2^E the leading power of the group's largest
+// input), bits = 62 - log2 sum|a| (and 4 less for the transform of d = 4, whose
+// two butterflies grow the values by 16), so that every sum is exact in 64
+// bits; the only other rounding is the final one to FP64. Error: at most
+// sum|a| 2^(E - bits) + half a unit in the last place, below that of the FP64
+// sum (a rounding of every partial sum). Returns false for groups whose
+// exponents leave [emin, emax] (infinities and NaNs among them).
+template <int D, int P, class Sink>
+__device__ __forceinline__ bool fixed_sum(const KParams& kp, const KsArgs& ka, const double (&x)[Pat<D, P>::M],
+                                          Sink&& sink) {
+  constexpr int M = Pat<D, P>::M;
+  unsigned mx = 0;
+#pragma unroll
+  for (int v = 0; v < M; v++) mx = max(mx, (unsigned)__double2hiint(x[v]) & 0x7FFFFFFFu);
+  unsigned E = mx & 0x7FF00000u;
+  if (E < ka.emin || E > ka.emax) {
+    unsigned any = mx;
+#pragma unroll
+    for (int v = 0; v < M; v++) any |= (unsigned)__double2loint(x[v]);
+    if (any != 0) return false;
+    E = ka.emin;  // a group of zeros is exact on any grid
+  }
+  // (E | 0xFFFFF) - |x|'s high word borrows nothing from the exponent field
+  const unsigned base = (E | 0xFFFFFu) + ((unsigned)(62 - ka.bits) << 20);
+  long long X[M];
+#pragma unroll
+  for (int v = 0; v < M; v++) {
+    const unsigned hi = (unsigned)__double2hiint(x[v]), lo = (unsigned)__double2loint(x[v]);
+    const unsigned k = (base - (hi & 0x7FFFFFFFu)) >> 20;
+    const unsigned long long mant =
+        (((unsigned long long)((hi & 0x000FFFFFu) | 0x00100000u) << 32) | lo) << 10;  // below 2^63
+    const long long q = (long long)((shr64(mant, k) + 1) >> 1);                       // rounded to the grid
+    X[v] = (int)hi < 0 ? -q : q;
+  }
+  const int sh = (int)(E >> 20) + ka.sh0;
+  if constexpr (D == 4 && wht_ok<P>()) {
+    constexpr int NB = M / 4, WOFF = wh_offset(P);
+    Fix64 t[M];
+#pragma unroll
+    for (int o = 0; o < NB; o++) {
+      const long long x0 = X[kWht<P>.orb[o][0]], x1 = X[kWht<P>.orb[o][1]], x2 = X[kWht<P>.orb[o][2]],
+                      x3 = X[kWht<P>.orb[o][3]];
+      const long long a0 = x0 + x1, a1 = x0 - x1, a2 = x2 + x3, a3 = x2 - x3;
+      t[4 * o] = fix64(a0 + a2);  // characters 0..3
+      t[4 * o + 1] = fix64(a1 + a3);
+      t[4 * o + 2] = fix64(a0 - a2);
+      t[4 * o + 3] = fix64(a1 - a3);
+    }
+#pragma unroll
+    for (int o = 0; o < NB; o++) {
+      long long yh[4] = {0, 0, 0, 0};
+#pragma unroll
+      for (int k = 0; k < 4; k++) {
+        const int i = 4 * o + k;
+#pragma unroll
+        for (int q = 0; q < 6; q++)
+          if (q < kWht<P>.nnz[i]) fix64_mac(yh[k], kp.wh[WOFF + kWht<P>.woff[i] + q], t[kWht<P>.col[i][q]]);
+      }
+      const long long b0 = yh[0] + yh[1], b1 = yh[0] - yh[1], b2 = yh[2] + yh[3], b3 = yh[2] - yh[3];
+      const long long y4[4] = {b0 + b2, b1 + b3, b0 - b2, b1 - b3};  // 4 Y
+#pragma unroll
+      for (int vi = 0; vi < 4; vi++) sink(kWht<P>.orb[o][vi], fixed_rn(y4[vi], sh - 2));
+    }
+  } else {
+    Fix64 t[M];
+    long long acc[M];
+#pragma unroll
+    for (int v = 0; v < M; v++) t[v] = fix64(X[v]);
+    if constexpr (P == 0) {
+#pragma unroll
+      for (int st = 0; st < MAXSTAGE_EXACT; st++) {
+        if (st >= kp.nci) break;
+        if (st > 0) {
+#pragma unroll
+          for (int u = 0; u < M; u++) t[u] = fix64(acc[u]);
+        }
+#pragma unroll
+        for (int u = 0; u < M; u++) acc[u] = 0;
+#pragma unroll
+        for (int s = 0; s < fact(D); s++) {
+          const int c = kp.ci[st][s];
+          if (c != 0) {
+#pragma unroll
+            for (int u = 0; u < M; u++) fix64_mac(acc[u], c, t[Pat<D, P>::idx(u, s)]);
+          }
+        }
+      }
+    } else {
+      const int* mp = kp.mp + mp_offset<D>(P);
+#pragma unroll
+      for (int u = 0; u < M; u++) {
+        acc[u] = 0;
+#pragma unroll
+        for (int v = 0; v < M; v++) fix64_mac(acc[u], mp[u * M + v], t[v]);
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < M; u++) sink(u, fixed_rn(acc[u], sh));
+  }
+  return true;
+}
+
+// shared-memory place of member u of the orbit with values val
+template <int D, int P>
+__device__ __forceinline__ int ks_slot(const KsArgs& ka, int u, const int (&val)[4]) {
+  int a = 0;
+#pragma unroll
+  for (int k = 0; k < D; k++) a += val[Pat<D, P>::lab(u, k)] * ka.pst[k];
+  return a;
+}
+
+// the FP64 reference order for one group, out of line: rare in AR_FIXED, and
+// inlined its FP64 instructions may be predicated into the common path
+template <int D, int P>
+static __device__ __noinline__ void ks_strict_group(const KParams& kp, const KsArgs& ka, unsigned tup, double* sm) {
+  constexpr int M = Pat<D, P>::M;
+  const int val[4] = {(int)(tup & 255), (int)(tup >> 8 & 255), (int)(tup >> 16 & 255), (int)(tup >> 24)};
+  double x[M];
+#pragma unroll
+  for (int u = 0; u < M; u++) x[u] = sm[ks_slot<D, P>(ka, u, val)];
+  strict_core<D, P>(kp, x);
+#pragma unroll
+  for (int u = 0; u < M; u++) sm[ks_slot<D, P>(ka, u, val)] = __dmul_rn(kp.alpha, x[u]);
+}
+
+template <int D, int P, int AR, typename T>
+__device__ __forceinline__ void ks_group(const KParams& kp, const KsArgs& ka, unsigned tup, T* sm) {
+  constexpr int M = Pat<D, P>::M;
+  const int val[4] = {(int)(tup & 255), (int)(tup >> 8 & 255), (int)(tup >> 16 & 255), (int)(tup >> 24)};
+  if constexpr (AR == AR_STRICT) {
+    ks_strict_group<D, P>(kp, ka, tup, sm);
+  } else {
+    T x[M];
+#pragma unroll
+    for (int u = 0; u < M; u++) x[u] = sm[ks_slot<D, P>(ka, u, val)];
+    if constexpr (AR == AR_FIXED) {
+      // (alpha not a power of two occurs for d <= 3 only: see ks_plan)
+      const bool mul = D <= 3 && (kp.flags & KF_ALPHA_MUL);
+      auto sink = [&](int u, double y) {
+        if (D <= 3 && mul) y = __dmul_rn(kp.alpha, y);
+        sm[ks_slot<D, P>(ka, u, val)] = y;
+      };
+      if (!fixed_sum<D, P>(kp, ka, x, sink)) ks_strict_group<D, P>(kp, ka, tup, sm);
+    } else {
+      T y[M];
+      apply_group<D, P, AR, T>(kp, x, y);
+#pragma unroll
+      for (int u = 0; u < M; u++) sm[ks_slot<D, P>(ka, u, val)] = y[u];
+    }
+  }
+}
+
+// every orbit of pattern P of the round's ns blocks; `first` is the table index
+// of the pattern's first tuple, `rot` spreads short patterns over the warps
+template <int D, int P, int AR, typename T>
+__device__ __forceinline__ void ks_pattern(const KParams& kp, const KsArgs& ka, const unsigned* tab, int ns, T* sm,
+                                           int& first, int& rot) {
+  const int n = (int)kp.norb[P];
+  const int total = n * ns;
+  int q = (int)threadIdx.x - rot;
+  if (q < 0) q += (int)blockDim.x;
+  for (; q < total; q += (int)blockDim.x) {
+    const int s = ns == 1 ? 0 : q / n;
+    ks_group<D, P, AR, T>(kp, ka, tab[first + q - s * n], sm + s * ka.Tp);
+  }
+  first += n;
+  rot = (rot + total) % (int)blockDim.x & ~31;
+}
+
+template <int D, int P>
+__device__ __forceinline__ void ks_table(const KParams& kp, unsigned* tab, int& first) {
+  const int n = (int)kp.norb[P];
+  for (int g = threadIdx.x; g < n; g += blockDim.x) {
+    int v[4] = {0, 0, 0, 0};
+    unrank<Pat<D, P>::ND>(g, kp.O, v);
+    tab[first + g] = (unsigned)v[0] | (unsigned)v[1] << 8 | (unsigned)v[2] << 16 | (unsigned)v[3] << 24;
+  }
+  first += n;
+}
+
+template <int D, int AR, int NT, int MINB, typename T>
+__global__ void __launch_bounds__(NT, MINB) ks_kernel(const __grid_constant__ KParams kp, const __grid_constant__ KsArgs ka) {
+  extern __shared__ __align__(16) unsigned char ks_smem[];
+  T* const sm = reinterpret_cast<T*>(ks_smem);
+  int64_t* const soff = reinterpret_cast<int64_t*>(ks_smem + ka.nspectab);  // [2][ns] spectator offsets of A and B
+  unsigned* const tab = reinterpret_cast<unsigned*>(soff + 2 * ka.ns);
+  {
+    int first = 0;
+    ks_table<D, 0>(kp, tab, first);
+    ks_table<D, 1>(kp, tab, first);
+    if constexpr (D >= 3) {
+      ks_table<D, 2>(kp, tab, first);
+      ks_table<D, 3>(kp, tab, first);
+    }
+    if constexpr (D == 4) {
+      ks_table<D, 4>(kp, tab, first);
+      ks_table<D, 5>(kp, tab, first);
+      ks_table<D, 6>(kp, tab, first);
+      ks_table<D, 7>(kp, tab, first);
+    }
+  }
+  const T* const A = static_cast<const T*>(kp.A);
+  T* const B = static_cast<T*>(kp.B);
+  // padded place of block element t
+  auto place = [&](int t) {
+    int f = t;
+    if (ka.pad) {
+      f += ks_div(t, ka.mO);
+      if constexpr (D >= 3) f += ks_div(t, ka.mO2);
+      if constexpr (D == 4) f += ks_div(t, ka.mO3);
+    }
+    return f;
+  };
+  const bool beta = kp.flags & KF_BETA;
+  const T bt = beta_of<T>(kp);
+  for (int64_t s0 = (int64_t)blockIdx.x * ka.ns; s0 < kp.S; s0 += (int64_t)gridDim.x * ka.ns) {
+    const int ns = (int)min((int64_t)ka.ns, kp.S - s0);
+    __syncthreads();  // the previous round's stores have read the blocks and offsets
+    for (int i = threadIdx.x; i < ns; i += NT) {
+      int64_t s = s0 + i, a = 0, b = 0;
+#pragma unroll
+      for (int k = 0; k < D; k++) {
+        const int64_t q = s / kp.sext[k], r = s - q * kp.sext[k];
+        a += r * kp.slda[k];
+        b += r * kp.sldb[k];
+        s = q;
+      }
+      soff[i] = a;
+      soff[ka.ns + i] = b;
+    }
+    __syncthreads();
+    const int ne = ns * ka.T;
+    for (int e = threadIdx.x; e < ne; e += NT) {
+      const int i = ka.ns == 1 ? 0 : ks_div(e, ka.mT);
+      const int t = e - i * ka.T;
+      cp_async<sizeof(T)>(sm + i * ka.Tp + place(t), A + soff[i] + t);
+    }
+    cp_async_commit();
+    cp_async_wait<0>();
+    __syncthreads();
+    int first = 0, rot = 0;
+    ks_pattern<D, 0, AR, T>(kp, ka, tab, ns, sm, first, rot);
+    ks_pattern<D, 1, AR, T>(kp, ka, tab, ns, sm, first, rot);
+    if constexpr (D >= 3) {
+      ks_pattern<D, 2, AR, T>(kp, ka, tab, ns, sm, first, rot);
+      ks_pattern<D, 3, AR, T>(kp, ka, tab, ns, sm, first, rot);
+    }
+    if constexpr (D == 4) {
+      ks_pattern<D, 4, AR, T>(kp, ka, tab, ns, sm, first, rot);
+      ks_pattern<D, 5, AR, T>(kp, ka, tab, ns, sm, first, rot);
+      ks_pattern<D, 6, AR, T>(kp, ka, tab, ns, sm, first, rot);
+      ks_pattern<D, 7, AR, T>(kp, ka, tab, ns, sm, first, rot);
+    }
+    __syncthreads();
+    if (beta) {
+      for (int e = threadIdx.x; e < ne; e += NT) {
+        const int i = ka.ns == 1 ? 0 : ks_div(e, ka.mT);
+        const int t = e - i * ka.T;
+        T* g = B + soff[ka.ns + i] + t;
+        *g = add_beta(sm[i * ka.Tp + place(t)], *g, bt);
+      }
+    } else {
+      for (int e = threadIdx.x; e < ne; e += NT) {
+        const int i = ka.ns == 1 ? 0 : ks_div(e, ka.mT);
+        const int t = e - i * ka.T;
+        B[soff[ka.ns + i] + t] = sm[i * ka.Tp + place(t)];
+      }
+    }
+  }
+}
+
+// most shared memory of a CTA
+constexpr int KS_SMEM_MAX = 227 * 1024 - 1024;
+// shared memory a round's blocks aim at: four CTAs per SM, so that one's copies
+// run under another's sums; larger blocks take one position per round and as many
+// CTAs as fit
+constexpr int KS_SMEM_AIM = 40 * 1024;
+
+// Whether the problem has KS's layout (permuted strides 1, O, .., O^(d-1) in
+// some order, the same in A and B) and its block fits on chip; fills ka and
+// the CTA's shared-memory bytes. Below O^d = 64 the rows are too short to be
+// worth staging, and FP64 with d = 4 needs the transform's weights (KF_WHT) for
+// AR_FIXED, else the FP64 order runs.
+inline bool ks_plan(int d, const KParams& kp, int es, KsArgs* ka, int* smem, bool* fixed) {
+  const int64_t O = kp.O;
+  int64_t T = 1;
+  for (int k = 0; k < d; k++) T *= O;
+  if (O < 2 || O > 255 || T < 64 || T > 40000) return false;
+  int rank[4] = {0, 0, 0, 0};
+  unsigned seen = 0;
+  for (int k = 0; k < d; k++) {
+    if (kp.lda[k] != kp.ldb[k]) return false;
+    int r = -1;
+    int64_t p = 1;
+    for (int q = 0; q < d; q++, p *= O)
+      if (kp.lda[k] == p) r = q;
+    if (r < 0 || (seen >> r & 1)) return false;
+    seen |= 1u << r;
+    rank[k] = r;
+  }
+  ka->pad = O % 2 == 0;
+  int64_t P[5] = {1, O + ka->pad, 0, 0, 0};
+  for (int q = 2; q <= d; q++) P[q] = O * P[q - 1] + ka->pad;
+  for (int k = 0; k < 4; k++) ka->pst[k] = k < d ? (int)P[rank[k]] : 0;
+  ka->T = (int)T;
+  ka->Tp = (int)P[d];
+  int64_t ntot = 0;
+  for (int p = 0; p < npatterns(d); p++) ntot += kp.norb[p];
+  ka->ntot = (int)ntot;
+  int64_t ns = KS_SMEM_AIM / (P[d] * es);
+  if (ns < 1) ns = 1;
+  if (ns > 64) ns = 64;
+  if (ns > 65535 / T) ns = 65535 / T > 0 ? 65535 / T : 1;  // ks_div's numerators
+  if (ns > kp.S) ns = kp.S;
+  ka->ns = (int)ns;
+  ka->nspectab = (int)((ns * P[d] * es + 15) / 16 * 16);
+  *smem = (int)(ka->nspectab + 16 * ns + 4 * ntot);
+  if (*smem > KS_SMEM_MAX) return false;
+  auto recip = [](int64_t n) { return (unsigned)(((1ull << 32) + n - 1) / n); };
+  ka->mT = recip(T);
+  ka->mO = recip(O);
+  ka->mO2 = recip(O * O);
+  ka->mO3 = d == 4 ? recip(O * O * O) : 0;
+  // AR_FIXED: the grid from the operator's 1-norm (chain: product of the factors')
+  *fixed = d <= 3 || (kp.flags & KF_WHT);
+  double L = 1;
+  for (int st = 0; st < kp.nci; st++) {
+    double n = 0;
+    for (int s = 0; s < (d == 2 ? 2 : (d == 3 ? 6 : 24)); s++) n += kp.ci[st][s] < 0 ? -kp.ci[st][s] : kp.ci[st][s];
+    L *= n;
+  }
+  int lg = 0;
+  while ((double)(1 << lg) < L) lg++;
+  ka->bits = 62 - lg - (d == 4 ? 4 : 0);
+  if (ka->bits > 60) ka->bits = 60;
+  // kp.cexp = (53 - 2 W + kdrop + aexp) << 20 + 0x80000, aexp = alpha's and the coefficients' scale
+  const int aexp = ((kp.cexp - 0x80000) >> 20) - 53 + 2 * kp.W - kp.kdrop;
+  ka->sh0 = -1023 - (ka->bits - 1) + aexp;
+  // the conversion's offsets 2^(1075 + sh - 2) .. 2^(1107 + sh) stay normal numbers
+  int lo = 3 - 1075 - ka->sh0, hi = 2040 - 1107 - ka->sh0;
+  if (lo < 72) lo = 72;  // subnormal inputs shift out entirely
+  if (hi > 2046) hi = 2046;
+  if (lo > hi) *fixed = false;
+  ka->emin = (unsigned)lo << 20;
+  ka->emax = (unsigned)hi << 20;
+  return true;
+}
+
+template <int D, int AR, int NT, int MINB, typename T>
+cudaError_t launch_ks_impl(const KParams& kp, const KsArgs& ka, int smem, cudaStream_t st) {
+  auto fn = ks_kernel<D, AR, NT, MINB, T>;
+  static DeviceCache cache;  // SMs, after raising the kernel's shared-memory limit
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  long long sms = 0;
+  const int rc = cache.get(dev, &sms, [&](long long* val) {
+    cudaError_t err = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, KS_SMEM_MAX);
+    if (err != cudaSuccess) return (int)err;
+    int n = 0;
+    err = cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+    *val = n;
+    return (int)err;
+  });
+  if (rc != 0) return rc < 0 ? cudaErrorInvalidDevice : (cudaError_t)rc;
+  const int64_t rounds = (kp.S + ka.ns - 1) / ka.ns;
+  int per = (KS_SMEM_MAX + 1024) / (smem + 1024);
+  if (per > MINB) per = MINB;
+  const int64_t grid = rounds < sms * per ? rounds : sms * per;
+  fn<<<(unsigned)grid, NT, smem, st>>>(kp, ka);
+  return cudaGetLastError();
+}
+
+// true (and *e the launch status) when KS takes the problem
+template <int D>
+bool launch_ks(const KParams& kp, int ar, cudaStream_t st, cudaError_t* e) {
+  KsArgs ka{};
+  int smem = 0;
+  bool fixed = false;
+  if (!ks_plan(D, kp, ar == AR_F32 ? 4 : 8, &ka, &smem, &fixed)) return false;
+  if constexpr (D == 4) {
+    // 24-member groups take 128 registers: two CTAs of 256 threads, or, where a
+    // block leaves room for one CTA only, one of 512
+    if (ar == AR_F32) *e = launch_ks_impl<4, AR_F32, 256, 2, float>(kp, ka, smem, st);
+    else if (!(ar == AR_EXACT && fixed)) *e = launch_ks_impl<4, AR_STRICT, 256, 2, double>(kp, ka, smem, st);
+    else if (smem > KS_SMEM_MAX / 2) *e = launch_ks_impl<4, AR_FIXED, 512, 1, double>(kp, ka, smem, st);
+    else *e = launch_ks_impl<4, AR_FIXED, 256, 2, double>(kp, ka, smem, st);
+  } else {
+    if (ar == AR_F32) *e = launch_ks_impl<D, AR_F32, 256, 5, float>(kp, ka, smem, st);
+    else if (ar == AR_EXACT && fixed) *e = launch_ks_impl<D, AR_FIXED, 256, 3, double>(kp, ka, smem, st);
+    else *e = launch_ks_impl<D, AR_STRICT, 256, 3, double>(kp, ka, smem, st);
+  }
+  return true;
+}
+
+}  // namespace ss
