@@ -11,7 +11,8 @@
 // unit-stride stores: each element crosses HBM once each way. The general
 // kernel KG reads and writes the same elements as scattered 8-byte accesses,
 // unranks a tuple per thread and sums with FP64 instructions: 2480 us on
-// A[32^3, 12^3], factorized Table II row 1 (0.37 TB/s), against 507 us here.
+// A[32^3, 12^3], factorized Table II row 1 (0.37 TB/s), against 470 us here (507 with one
+// buffer per CTA).
 //
 // - Canonical tuples come from a table in shared memory, grouped by equality
 //   pattern and built once per CTA, so warps run one pattern's code and no
@@ -34,18 +35,20 @@ constexpr int AR_FIXED = 4;  // kernel-template choice of this file: FP64 throug
 struct KsArgs {
   int ns;             // spectator positions per round
   int T, Tp;          // elements of a permuted block, and with its padding
+  int nbuf;           // buffers of ns blocks (2: the next round is copied under the sums)
   unsigned mT, mO;    // ceil(2^32 / T), ceil(2^32 / O)
   unsigned mO2, mO3;  // ceil(2^32 / O^2), ceil(2^32 / O^3)
+  unsigned mN[8];     // ceil(2^32 / orbits of pattern p)
   int pad;            // 1: padded rows, planes, volumes (even O)
   int pst[4];         // shared-memory stride of permuted index k
   int ntot;           // canonical tuples
-  int nspectab;       // offset of the spectator-offset table in shared memory (bytes)
+  int otab;           // offset of the tables in shared memory (bytes)
   int bits;           // AR_FIXED: an input's magnitude stays below 2^bits
   int sh0;            // AR_FIXED: result exponent offset (see fixed_sum)
   unsigned emin, emax;
 };
 
-// quotient by a constant with its precomputed reciprocal (numerators below 2^16)
+// quotient by a constant n > 1 with its precomputed reciprocal (numerators below 2^16)
 __device__ __forceinline__ int ks_div(int n, unsigned m) { return (int)__umulhi((unsigned)n, m); }
 
 // A fixed-point value lo + hi 2^32 with a SIGNED low word, so that a product
@@ -237,7 +240,7 @@ __device__ __forceinline__ void ks_pattern(const KParams& kp, const KsArgs& ka, 
   int q = (int)threadIdx.x - rot;
   if (q < 0) q += (int)blockDim.x;
   for (; q < total; q += (int)blockDim.x) {
-    const int s = ns == 1 ? 0 : q / n;
+    const int s = n == 1 ? q : ks_div(q, ka.mN[P]);
     ks_group<D, P, AR, T>(kp, ka, tab[first + q - s * n], sm + s * ka.Tp);
   }
   first += n;
@@ -258,9 +261,12 @@ __device__ __forceinline__ void ks_table(const KParams& kp, unsigned* tab, int& 
 template <int D, int AR, int NT, int MINB, typename T>
 __global__ void __launch_bounds__(NT, MINB) ks_kernel(const __grid_constant__ KParams kp, const __grid_constant__ KsArgs ka) {
   extern __shared__ __align__(16) unsigned char ks_smem[];
-  T* const sm = reinterpret_cast<T*>(ks_smem);
-  int64_t* const soff = reinterpret_cast<int64_t*>(ks_smem + ka.nspectab);  // [2][ns] spectator offsets of A and B
-  unsigned* const tab = reinterpret_cast<unsigned*>(soff + 2 * ka.ns);
+  T* const buf = reinterpret_cast<T*>(ks_smem);
+  // tables: spectator offsets of A and B [3][2][ns] (the round that is stored, the
+  // one that is summed and the one that is copied), canonical tuples, padded places
+  int64_t* const soff = reinterpret_cast<int64_t*>(ks_smem + ka.otab);
+  unsigned* const tab = reinterpret_cast<unsigned*>(soff + 6 * ka.ns);
+  unsigned short* const place = reinterpret_cast<unsigned short*>(tab + ka.ntot);
   {
     int first = 0;
     ks_table<D, 0>(kp, tab, first);
@@ -276,24 +282,21 @@ __global__ void __launch_bounds__(NT, MINB) ks_kernel(const __grid_constant__ KP
       ks_table<D, 7>(kp, tab, first);
     }
   }
-  const T* const A = static_cast<const T*>(kp.A);
-  T* const B = static_cast<T*>(kp.B);
   // padded place of block element t
-  auto place = [&](int t) {
+  for (int t = threadIdx.x; t < ka.T; t += NT) {
     int f = t;
     if (ka.pad) {
       f += ks_div(t, ka.mO);
       if constexpr (D >= 3) f += ks_div(t, ka.mO2);
       if constexpr (D == 4) f += ks_div(t, ka.mO3);
     }
-    return f;
-  };
-  const bool beta = kp.flags & KF_BETA;
-  const T bt = beta_of<T>(kp);
-  for (int64_t s0 = (int64_t)blockIdx.x * ka.ns; s0 < kp.S; s0 += (int64_t)gridDim.x * ka.ns) {
-    const int ns = (int)min((int64_t)ka.ns, kp.S - s0);
-    __syncthreads();  // the previous round's stores have read the blocks and offsets
-    for (int i = threadIdx.x; i < ns; i += NT) {
+    place[t] = (unsigned short)f;
+  }
+  const T* const A = static_cast<const T*>(kp.A);
+  T* const B = static_cast<T*>(kp.B);
+  const int64_t step = (int64_t)gridDim.x * ka.ns;
+  auto offsets = [&](int64_t s0, int64_t* so) {
+    for (int i = threadIdx.x; i < ka.ns && s0 + i < kp.S; i += NT) {
       int64_t s = s0 + i, a = 0, b = 0;
 #pragma unroll
       for (int k = 0; k < D; k++) {
@@ -302,18 +305,52 @@ __global__ void __launch_bounds__(NT, MINB) ks_kernel(const __grid_constant__ KP
         b += r * kp.sldb[k];
         s = q;
       }
-      soff[i] = a;
-      soff[ka.ns + i] = b;
+      so[i] = a;
+      so[ka.ns + i] = b;
     }
-    __syncthreads();
-    const int ne = ns * ka.T;
-    for (int e = threadIdx.x; e < ne; e += NT) {
-      const int i = ka.ns == 1 ? 0 : ks_div(e, ka.mT);
-      const int t = e - i * ka.T;
-      cp_async<sizeof(T)>(sm + i * ka.Tp + place(t), A + soff[i] + t);
+  };
+  auto count = [&](int64_t s0) { return (int)min((int64_t)ka.ns, kp.S - s0); };
+  // f(block of the round, element of the block): by whole blocks where they fill the CTA
+  auto each = [&](int ns, auto&& f) {
+    if (ka.T >= 4 * NT) {
+      for (int i = 0; i < ns; i++)
+        for (int t = threadIdx.x; t < ka.T; t += NT) f(i, t);
+    } else {
+      const int ne = ns * ka.T;
+      for (int e = threadIdx.x; e < ne; e += NT) {
+        const int i = ka.ns == 1 ? 0 : ks_div(e, ka.mT);
+        f(i, e - i * ka.T);
+      }
     }
+  };
+  auto load = [&](int ns, T* sm, const int64_t* so) {
+    each(ns, [&](int i, int t) { cp_async<sizeof(T)>(sm + i * ka.Tp + place[t], A + so[i] + t); });
+  };
+  const bool beta = kp.flags & KF_BETA;
+  const T bt = beta_of<T>(kp);
+  int64_t s0 = (int64_t)blockIdx.x * ka.ns;
+  offsets(s0, soff);
+  __syncthreads();
+  if (ka.nbuf == 2) {
+    load(count(s0), buf, soff);
     cp_async_commit();
-    cp_async_wait<0>();
+  }
+  for (int k = 0; s0 < kp.S; s0 += step, k++) {
+    const int ns = count(s0);
+    T* const sm = buf + (ka.nbuf == 2 && (k & 1) ? ka.ns * ka.Tp : 0);
+    int64_t* const so = soff + k % 3 * 2 * ka.ns;
+    int64_t* const son = soff + (k + 1) % 3 * 2 * ka.ns;
+    offsets(s0 + step, son);
+    if (ka.nbuf == 2) {
+      __syncthreads();  // the next offsets are there; the previous round's stores have read the other buffer
+      if (s0 + step < kp.S) load(count(s0 + step), buf + ((k & 1) ? 0 : ka.ns * ka.Tp), son);
+      cp_async_commit();
+      cp_async_wait<1>();
+    } else {
+      load(ns, sm, so);
+      cp_async_commit();
+      cp_async_wait<0>();
+    }
     __syncthreads();
     int first = 0, rot = 0;
     ks_pattern<D, 0, AR, T>(kp, ka, tab, ns, sm, first, rot);
@@ -329,29 +366,22 @@ __global__ void __launch_bounds__(NT, MINB) ks_kernel(const __grid_constant__ KP
       ks_pattern<D, 7, AR, T>(kp, ka, tab, ns, sm, first, rot);
     }
     __syncthreads();
-    if (beta) {
-      for (int e = threadIdx.x; e < ne; e += NT) {
-        const int i = ka.ns == 1 ? 0 : ks_div(e, ka.mT);
-        const int t = e - i * ka.T;
-        T* g = B + soff[ka.ns + i] + t;
-        *g = add_beta(sm[i * ka.Tp + place(t)], *g, bt);
-      }
-    } else {
-      for (int e = threadIdx.x; e < ne; e += NT) {
-        const int i = ka.ns == 1 ? 0 : ks_div(e, ka.mT);
-        const int t = e - i * ka.T;
-        B[soff[ka.ns + i] + t] = sm[i * ka.Tp + place(t)];
-      }
-    }
+    if (beta)
+      each(ns, [&](int i, int t) {
+        T* g = B + so[ka.ns + i] + t;
+        *g = add_beta(sm[i * ka.Tp + place[t]], *g, bt);
+      });
+    else
+      each(ns, [&](int i, int t) { B[so[ka.ns + i] + t] = sm[i * ka.Tp + place[t]]; });
+    if (ka.nbuf == 1) __syncthreads();  // the buffer is free again
   }
 }
 
 // most shared memory of a CTA
 constexpr int KS_SMEM_MAX = 227 * 1024 - 1024;
-// shared memory a round's blocks aim at: four CTAs per SM, so that one's copies
-// run under another's sums; larger blocks take one position per round and as many
-// CTAs as fit
-constexpr int KS_SMEM_AIM = 40 * 1024;
+// shared memory a round's blocks aim at: three CTAs per SM with two buffers each;
+// larger blocks take one position per round, and one buffer where two do not fit
+constexpr int KS_SMEM_AIM = 32 * 1024;
 
 // Whether the problem has KS's layout (permuted strides 1, O, .., O^(d-1) in
 // some order, the same in A and B) and its block fits on chip; fills ka and
@@ -390,9 +420,17 @@ inline bool ks_plan(int d, const KParams& kp, int es, KsArgs* ka, int* smem, boo
   if (ns > 65535 / T) ns = 65535 / T > 0 ? 65535 / T : 1;  // ks_div's numerators
   if (ns > kp.S) ns = kp.S;
   ka->ns = (int)ns;
-  ka->nspectab = (int)((ns * P[d] * es + 15) / 16 * 16);
-  *smem = (int)(ka->nspectab + 16 * ns + 4 * ntot);
-  if (*smem > KS_SMEM_MAX) return false;
+  if (P[d] > 65535) return false;  // 16-bit places
+  const int64_t tables = 48 * ns + 4 * ntot + (2 * T + 15) / 16 * 16;
+  for (ka->nbuf = 2; ka->nbuf >= 1; ka->nbuf--) {
+    ka->otab = (int)((ka->nbuf * ns * P[d] * es + 15) / 16 * 16);
+    *smem = (int)(ka->otab + tables);
+    if (*smem <= KS_SMEM_MAX) break;
+  }
+  if (ka->nbuf == 0) return false;
+  for (int p = 0; p < 8; p++) ka->mN[p] = 0;
+  for (int p = 0; p < npatterns(d); p++)
+    if (kp.norb[p] > 0) ka->mN[p] = (unsigned)(((1ull << 32) + kp.norb[p] - 1) / kp.norb[p]);
   auto recip = [](int64_t n) { return (unsigned)(((1ull << 32) + n - 1) / n); };
   ka->mT = recip(T);
   ka->mO = recip(O);
