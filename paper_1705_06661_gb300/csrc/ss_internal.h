@@ -345,6 +345,10 @@ constexpr int MP_MAX = MP_TOTAL_4;
 #ifndef SS_K1_KBMAX4
 #define SS_K1_KBMAX4 1
 #endif
+// K1, FP32 with 4-byte loads, d <= 3: chunks a thread takes at a time for the generic orbit
+#ifndef SS_K1_KB0F32
+#define SS_K1_KB0F32 2
+#endif
 // K1, d = 4 transform path: spectator positions per member per block
 #ifndef SS_K1_POS4
 #define SS_K1_POS4 5120

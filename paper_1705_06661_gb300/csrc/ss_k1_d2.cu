@@ -4,17 +4,16 @@
 namespace ss {
 
 cudaError_t launch_k1_d2(const KParams& kp, int ar, int vec, cudaStream_t st) {
-  const dim3 grid((unsigned)kp.pre[npatterns(2)]), block(256);
   if (ar == AR_EXACT) {
-    if (vec == 2) k1_kernel<2, AR_EXACT, 2, double><<<grid, block, 0, st>>>(kp);
-    else k1_kernel<2, AR_EXACT, 1, double><<<grid, block, 0, st>>>(kp);
+    if (vec == 2) launch_k1_bt<2, AR_EXACT, 2, double>(kp, st);
+    else launch_k1_bt<2, AR_EXACT, 1, double>(kp, st);
   } else if (ar == AR_STRICT) {
-    if (vec == 2) k1_kernel<2, AR_STRICT, 2, double><<<grid, block, 0, st>>>(kp);
-    else k1_kernel<2, AR_STRICT, 1, double><<<grid, block, 0, st>>>(kp);
+    if (vec == 2) launch_k1_bt<2, AR_STRICT, 2, double>(kp, st);
+    else launch_k1_bt<2, AR_STRICT, 1, double>(kp, st);
   } else {
-    if (vec == 4) k1_kernel<2, AR_F32, 4, float><<<grid, block, 0, st>>>(kp);
-    else if (vec == 2) k1_kernel<2, AR_F32, 2, float><<<grid, block, 0, st>>>(kp);
-    else k1_kernel<2, AR_F32, 1, float><<<grid, block, 0, st>>>(kp);
+    if (vec == 4) launch_k1_bt<2, AR_F32, 4, float>(kp, st);
+    else if (vec == 2) launch_k1_bt<2, AR_F32, 2, float>(kp, st);
+    else launch_k1_bt<2, AR_F32, 1, float>(kp, st);
   }
   return cudaGetLastError();
 }

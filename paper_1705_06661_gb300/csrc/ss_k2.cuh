@@ -176,7 +176,7 @@ __device__ __forceinline__ void k2_group(const KParams& kp, const int (&w)[4], T
 #pragma unroll
     for (int u = 0; u < M; u++) x[u] = sm[slot(u)];
     if constexpr (wht_ok<EP>()) {
-      auto sink = [&](int u, double v) { sm[slot(u)] = v; };
+      auto sink = [&](int u, double v, int) { sm[slot(u)] = v; };
       if (!exact_core_wht4<EP>(kp, x, sink)) k2_strict_group<D, BP, EP>(kp, w, sm);
     } else {
       T y[M];

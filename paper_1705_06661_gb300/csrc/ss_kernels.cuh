@@ -304,9 +304,15 @@ __device__ __forceinline__ bool exact_core_grouped4(const KParams& kp, const dou
 // are joined in 64 bits and the inverse transform (the same butterflies)
 // gives 4 Y, Y the integer sum sum_v M[u][v] X_v of the dense core. Rounding
 // off kdrop + 2 bits of 4 Y is rounding off kdrop bits of Y, so outputs are
-// bit-identical to exact_core on the same grid. Outputs go to sink(u, y).
-template <int P, class Sink>
-__device__ __forceinline__ bool exact_core_wht4(const KParams& kp, const double (&x)[Pat<4, P>::M], Sink&& sink) {
+// bit-identical to exact_core on the same grid. Outputs go to sink(u, y, vi),
+// those of V-orbit o (vi = 0..3) after a call of pre(o).
+struct NoPre {
+  __device__ __forceinline__ void operator()(int) const {}
+};
+
+template <int P, class Sink, class Pre = NoPre>
+__device__ __forceinline__ bool exact_core_wht4(const KParams& kp, const double (&x)[Pat<4, P>::M], Sink&& sink,
+                                                Pre&& pre = Pre()) {
   constexpr int M = Pat<4, P>::M, NB = M / 4;
   constexpr int WOFF = wh_offset(P);
   unsigned E = 0;
@@ -349,6 +355,7 @@ __device__ __forceinline__ bool exact_core_wht4(const KParams& kp, const double 
   const long long r4 = kp.rnd << 2;
 #pragma unroll
   for (int o = 0; o < NB; o++) {
+    pre(o);
     long long yh[4];
 #pragma unroll
     for (int k = 0; k < 4; k++) {
@@ -369,7 +376,7 @@ __device__ __forceinline__ bool exact_core_wht4(const KParams& kp, const double 
 #pragma unroll
     for (int vi = 0; vi < 4; vi++) {
       const long long Y = (y4[vi] + r4) >> sh;
-      sink(kWht<P>.orb[o][vi], fixed_to_double_fp64(Y, chi, C));
+      sink(kWht<P>.orb[o][vi], fixed_to_double_fp64(Y, chi, C), vi);
     }
   }
   return true;
@@ -434,6 +441,14 @@ __device__ __forceinline__ T beta_of(const KParams& kp) {
 // B = alpha S(A) + beta B_old: the beta term, in the reference order for FP64
 __device__ __forceinline__ double add_beta(double y, double b, double beta) { return __dadd_rn(y, __dmul_rn(beta, b)); }
 __device__ __forceinline__ float add_beta(float y, float b, float beta) { return fmaf(beta, b, y); }
+
+// the same after the exact core, whose result is not the reference's rounding anyway:
+// one FP64 instruction and one rounding less
+template <int AR, typename T>
+__device__ __forceinline__ T add_beta_of(T y, T b, T beta) {
+  if constexpr (AR == AR_EXACT) return fma(beta, b, y);
+  else return add_beta(y, b, beta);
+}
 
 template <typename T, int VEC>
 struct VecT;
@@ -520,17 +535,27 @@ static __device__ __noinline__ void scaled_generic4(const KParams& kp, const int
   auto sink = [&](int u, double v) {
     double* dst = B + offB[u] + s;
     v = __dmul_rn(kp.alpha, v);
-    if (beta) v = add_beta(v, *dst, kp.beta);
+    if (beta) v = fma(kp.beta, *dst, v);
     *dst = v;
   };
   if (!exact_core_grouped4<SS_4D_GROUPS>(kp, x, sink)) strict_fallback_generic4(kp, offA, offB, s);
 }
 
-// chunks a K1 thread takes at a time for an orbit of m members: the generic
-// orbit's d! over m, at most kbmax
-constexpr int k1_batch(int D, int m, int kbmax) {
-  return m >= fact(D) ? 1 : (fact(D) / m < kbmax ? fact(D) / m : kbmax);
+// chunks a K1 thread takes at a time for an orbit of m members: kb0 times the
+// generic orbit's d! over m, this at most kbmax
+constexpr int k1_batch(int D, int m, int kbmax, int kb0 = 1) {
+  return kb0 * (m >= fact(D) ? 1 : (fact(D) / m < kbmax ? fact(D) / m : kbmax));
 }
+
+// kb0 of the single-problem kernel: FP32 runs that allow no 16-byte loads (odd
+// extents) take two chunks, so that a thread has more loads in flight
+template <int D, int AR, int VEC>
+constexpr int k1_kb0() {
+  return AR == AR_F32 && D <= 3 && VEC == 1 ? SS_K1_KB0F32 : 1;
+}
+
+// asks L2 for the line of B that the beta term will read after the sums
+__device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 
 // ---------------------------------------------------------------------------
 // K1 body for pattern P. Warp 0 unranks the orbit and writes the m member
@@ -541,8 +566,9 @@ constexpr int k1_batch(int D, int m, int kbmax) {
 // XW selects the Klein four-group path of d = 4 exact orbits: 0 never, 1 for
 // every transformable pattern (the planner set KF_WHT), 2 when the problem's
 // KF_WHT flag says so (batched kernels, whose problems differ).
-// KBM: the most chunks a thread takes at a time (k1_batch).
-template <int D, int P, int AR, int VEC, typename T, int NST = 0, int XW = 0, int KBM = 1>
+// KBM, KB0: chunks a thread takes at a time (k1_batch). BT: the beta term never
+// (0), always (1) or by the problem's flag (2).
+template <int D, int P, int AR, int VEC, typename T, int NST = 0, int XW = 0, int KBM = 1, int KB0 = 1, int BT = 2>
 __device__ __forceinline__ void k1_body(const KParams& kp, int64_t orb, int64_t c0, int64_t c1) {
   constexpr int M = Pat<D, P>::M;
   __shared__ int64_t soff[2][24];
@@ -571,7 +597,7 @@ __device__ __forceinline__ void k1_body(const KParams& kp, int64_t orb, int64_t 
   const int64_t step = (int64_t)blockDim.x * VEC;
   if constexpr (D == 4 && AR == AR_EXACT && VEC == 1 && XW != 0) {
     if (XW == 1 || (kp.flags & KF_WHT)) {
-      const bool beta = kp.flags & KF_BETA;
+      const bool beta = BT == 1 || (kp.flags & KF_BETA);
       constexpr int KB = k1_batch(D, M, KBM);
       for (int64_t c = c0; c < c1; c += KB) {
         if constexpr (SS_4DW_PREFETCH) {
@@ -608,6 +634,10 @@ __device__ __forceinline__ void k1_body(const KParams& kp, int64_t orb, int64_t 
           if (ok[k]) {
 #pragma unroll
             for (int u = 0; u < M; u++) x[k][u] = A[soff[0][u] + sk[k]];
+            if constexpr (BT == 1) {
+#pragma unroll
+              for (int u = 0; u < M; u++) prefetch_l2(B + soff[1][u] + sk[k]);
+            }
           }
 #pragma unroll
         for (int k = 0; k < KB; k++) {
@@ -615,11 +645,24 @@ __device__ __forceinline__ void k1_body(const KParams& kp, int64_t orb, int64_t 
           const int64_t s = sk[k];
           auto sink = [&](int u, double v) {
             T* dst = B + soff[1][u] + s;
-            if (beta) v = add_beta(v, *dst, kp.beta);
+            if (beta) v = fma(kp.beta, *dst, v);
             *dst = v;
           };
           if constexpr (wht_ok<P>()) {
-            if (!exact_core_wht4<P>(kp, x[k], sink)) strict_fallback4<P>(kp, soff[0], soff[1], s);
+            if constexpr (BT == 1) {
+              // a V-orbit's four old values are loaded together, ahead of its sums
+              // (a load behind a store that may alias it waits for its own round trip)
+              double old[4];
+              auto pre = [&](int o) {
+#pragma unroll
+                for (int vi = 0; vi < 4; vi++) old[vi] = B[soff[1][kWht<P>.orb[o][vi]] + s];
+              };
+              auto sink4 = [&](int u, double v, int vi) { B[soff[1][u] + s] = fma(kp.beta, old[vi], v); };
+              if (!exact_core_wht4<P>(kp, x[k], sink4, pre)) strict_fallback4<P>(kp, soff[0], soff[1], s);
+            } else {
+              auto sink2 = [&](int u, double v, int) { sink(u, v); };
+              if (!exact_core_wht4<P>(kp, x[k], sink2)) strict_fallback4<P>(kp, soff[0], soff[1], s);
+            }
           } else {
             // the two patterns V does not act on freely: the dense core on the
             // same grid, with the strict core out of line (inlined, the compiler
@@ -640,7 +683,7 @@ __device__ __forceinline__ void k1_body(const KParams& kp, int64_t orb, int64_t 
   // orbits with fewer members than the generic one take KB chunks at a time,
   // so that every thread has about the same number of loads in flight
   constexpr bool G4 = D == 4 && P == 0 && AR == AR_EXACT && VEC == 1;
-  constexpr int KB = G4 ? 1 : k1_batch(D, M, KBM);
+  constexpr int KB = G4 ? 1 : k1_batch(D, M, KBM, KB0);
   for (int64_t c0k = c0; c0k < c1; c0k += KB) {
     int64_t sk[KB];
     bool ok[KB];
@@ -669,22 +712,30 @@ __device__ __forceinline__ void k1_body(const KParams& kp, int64_t orb, int64_t 
           for (int e = 0; e < VEC; e++) xk[k][e][u] = v[e];
         }
       }
+    if constexpr (BT == 1) {
+#pragma unroll
+      for (int k = 0; k < KB; k++)
+        if (ok[k]) {
+#pragma unroll
+          for (int u = 0; u < M; u++) prefetch_l2(B + soff[1][u] + sk[k]);
+        }
+    }
     if constexpr (G4) {
       auto& x = xk[0];
-      const bool beta = kp.flags & KF_BETA;
+      const bool beta = BT == 2 ? (kp.flags & KF_BETA) != 0 : BT == 1;
       bool done;
       if (!SS_4D_SCALED_OUTOFLINE && (kp.flags & KF_ALPHA_MUL)) {
         auto sink = [&](int u, double v) {
           T* dst = B + soff[1][u] + s;
           v = __dmul_rn(kp.alpha, v);
-          if (beta) v = add_beta(v, *dst, kp.beta);
+          if (beta) v = fma(kp.beta, *dst, v);
           *dst = v;
         };
         done = exact_core_grouped4<SS_4D_GROUPS>(kp, x[0], sink);
       } else {
         auto sink = [&](int u, double v) {
           T* dst = B + soff[1][u] + s;
-          if (beta) v = add_beta(v, *dst, kp.beta);
+          if (beta) v = fma(kp.beta, *dst, v);
           *dst = v;
         };
         done = exact_core_grouped4<SS_4D_GROUPS>(kp, x[0], sink);
@@ -692,7 +743,7 @@ __device__ __forceinline__ void k1_body(const KParams& kp, int64_t orb, int64_t 
       if (!done) strict_fallback_generic4(kp, soff[0], soff[1], s);
       continue;
     }
-    const bool beta = kp.flags & KF_BETA;
+    const bool beta = BT == 2 ? (kp.flags & KF_BETA) != 0 : BT == 1;
     const T bt = beta_of<T>(kp);
 #pragma unroll
     for (int k = 0; k < KB; k++) {
@@ -700,14 +751,25 @@ __device__ __forceinline__ void k1_body(const KParams& kp, int64_t orb, int64_t 
       T y[VEC][M];
 #pragma unroll
       for (int e = 0; e < VEC; e++) apply_group<D, P, AR, T, NST>(kp, xk[k][e], y[e]);
+      if (BT == 1) {
+        // every old value before the first store: a load behind a store that may
+        // alias it waits for its own round trip, m of them in a row
+        T o[M][VEC];
+#pragma unroll
+        for (int u = 0; u < M; u++) vload<T, VEC>(B + soff[1][u] + sk[k], o[u]);
+#pragma unroll
+        for (int u = 0; u < M; u++)
+#pragma unroll
+          for (int e = 0; e < VEC; e++) y[e][u] = add_beta_of<AR>(y[e][u], o[u][e], bt);
+      }
 #pragma unroll
       for (int u = 0; u < M; u++) {
         T v[VEC];
         T* dst = B + soff[1][u] + sk[k];
-        if (beta) {
+        if (BT == 2 && beta) {
           vload<T, VEC>(dst, v);
 #pragma unroll
-          for (int e = 0; e < VEC; e++) v[e] = add_beta(y[e][u], v[e], bt);
+          for (int e = 0; e < VEC; e++) v[e] = add_beta_of<AR>(y[e][u], v[e], bt);
         } else {
 #pragma unroll
           for (int e = 0; e < VEC; e++) v[e] = y[e][u];
@@ -729,7 +791,7 @@ __device__ __forceinline__ int find_pattern(const int64_t* pre, int64_t b) {
 
 // one K1 block of work: block index b of the problem's grid -> (pattern,
 // orbit, chunk range)
-template <int D, int AR, int VEC, typename T, int XW = 0, int KBM = 1>
+template <int D, int AR, int VEC, typename T, int XW = 0, int KBM = 1, int KB0 = 1, int BT = 2>
 __device__ __forceinline__ void k1_block(const KParams& kp, int64_t b) {
   const int p = find_pattern<D>(kp.pre, b);
   const int64_t bpo = (kp.nchunk + kp.cpb - 1) / kp.cpb;  // blocks per orbit
@@ -739,26 +801,35 @@ __device__ __forceinline__ void k1_block(const KParams& kp, int64_t b) {
   const int64_t c0 = cb * kp.cpb;
   const int64_t c1 = min(kp.nchunk, c0 + kp.cpb);
   switch (p) {
-    case 0: k1_body<D, 0, AR, VEC, T, 0, XW, KBM>(kp, orb, c0, c1); break;
-    case 1: k1_body<D, 1, AR, VEC, T, 0, XW, KBM>(kp, orb, c0, c1); break;
-    case 2: if constexpr (npatterns(D) > 2) k1_body<D, 2, AR, VEC, T, 0, XW, KBM>(kp, orb, c0, c1); break;
-    case 3: if constexpr (npatterns(D) > 3) k1_body<D, 3, AR, VEC, T, 0, XW, KBM>(kp, orb, c0, c1); break;
+    case 0: k1_body<D, 0, AR, VEC, T, 0, XW, KBM, KB0, BT>(kp, orb, c0, c1); break;
+    case 1: k1_body<D, 1, AR, VEC, T, 0, XW, KBM, KB0, BT>(kp, orb, c0, c1); break;
+    case 2: if constexpr (npatterns(D) > 2) k1_body<D, 2, AR, VEC, T, 0, XW, KBM, KB0, BT>(kp, orb, c0, c1); break;
+    case 3: if constexpr (npatterns(D) > 3) k1_body<D, 3, AR, VEC, T, 0, XW, KBM, KB0, BT>(kp, orb, c0, c1); break;
     default:
       if constexpr (D == 4) {
         switch (p) {
-          case 4: k1_body<D, 4, AR, VEC, T, 0, XW, KBM>(kp, orb, c0, c1); break;
-          case 5: k1_body<D, 5, AR, VEC, T, 0, XW, KBM>(kp, orb, c0, c1); break;
-          case 6: k1_body<D, 6, AR, VEC, T, 0, XW, KBM>(kp, orb, c0, c1); break;
-          case 7: k1_body<D, 7, AR, VEC, T, 0, XW, KBM>(kp, orb, c0, c1); break;
+          case 4: k1_body<D, 4, AR, VEC, T, 0, XW, KBM, KB0, BT>(kp, orb, c0, c1); break;
+          case 5: k1_body<D, 5, AR, VEC, T, 0, XW, KBM, KB0, BT>(kp, orb, c0, c1); break;
+          case 6: k1_body<D, 6, AR, VEC, T, 0, XW, KBM, KB0, BT>(kp, orb, c0, c1); break;
+          case 7: k1_body<D, 7, AR, VEC, T, 0, XW, KBM, KB0, BT>(kp, orb, c0, c1); break;
         }
       }
   }
 }
 
-template <int D, int AR, int VEC, typename T, int XW = 0>
+template <int D, int AR, int VEC, typename T, int XW = 0, int BT = 2>
 __global__ void __launch_bounds__(256, (D == 4 && AR == AR_EXACT) ? (XW ? SS_4DW_MINBLOCKS : SS_4D_MINBLOCKS) : 1)
     k1_kernel(const __grid_constant__ KParams kp) {
-  k1_block<D, AR, VEC, T, XW, D <= 3 ? SS_K1_KBMAX3 : SS_K1_KBMAX4>(kp, blockIdx.x);
+  k1_block<D, AR, VEC, T, XW, D <= 3 ? SS_K1_KBMAX3 : SS_K1_KBMAX4, k1_kb0<D, AR, VEC>(), BT>(kp, blockIdx.x);
+}
+
+// single problems: with and without the beta term as two kernels (in one,
+// the old values' registers cost the beta = 0 path a resident CTA)
+template <int D, int AR, int VEC, typename T>
+void launch_k1_bt(const KParams& kp, cudaStream_t st) {
+  const dim3 grid((unsigned)kp.pre[npatterns(D)]), block(256);
+  if (kp.flags & KF_BETA) k1_kernel<D, AR, VEC, T, 0, 1><<<grid, block, 0, st>>>(kp);
+  else k1_kernel<D, AR, VEC, T, 0, 0><<<grid, block, 0, st>>>(kp);
 }
 
 // ---------------------------------------------------------------------------
