@@ -3,7 +3,11 @@
 
 namespace ss {
 
+bool launch_k2t_d4(const KParams& kp, int ar, cudaStream_t st, cudaError_t* e);
+
 cudaError_t launch_k2_d4_exact(const KParams& kp, cudaStream_t st) {
+  cudaError_t e;
+  if (launch_k2t_d4(kp, AR_EXACT, st, &e)) return e;  // 16-byte strides, no beta term
   if (kp.flags & KF_WHT) return launch_k2_impl<4, AR_EXACT_XW, double>(kp, st);
   return launch_k2_impl<4, AR_EXACT, double>(kp, st);
 }
