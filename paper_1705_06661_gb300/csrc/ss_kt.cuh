@@ -10,14 +10,15 @@
 // exact: the splitting of Ozaki, Ogita, Oishi and Rump ("Error-free
 // transformations of matrix multiplication", Numer. Algorithms 59, 2012).
 //
-// - The tuples t are taken in chunks of 144. Per chunk, a row s of S(A) and a
+// - The tuples t are taken in chunks of 192. Per chunk, a row s of S(A) and a
 //   column y of W each get one power-of-two scale (from the largest |A| resp. |W|
 //   of the chunk) and become 55-bit signed integers v = sum_i d_i 256^(6-i),
 //   i = 0..6, -128 <= d_i <= 127. The orbit operator runs on the integers of A
 //   (two limbs of 24 and up to 26 bits, 32-bit multiply-adds): S(A) is exact on
 //   the grid 2^(E + 1 - bits), bits = 54 - log2 sum|a|.
-// - D_d = sum over t and i + j = d of d_i(A) d_j(W), d = 0..6: at most
-//   7 * 144 products of magnitude at most 2^14, below 2^24, so exact in FP32.
+// - D_d = sum over t and i + j = d of d_i(A) d_j(W), d = 0..6. Leading digits are at
+//   most 64, so |D_d| <= 192 d 2^14: below 2^24, hence exact in FP32, for d <= 5; D_6
+//   may round above 2^24, by a unit 2^-8 of the smallest that is kept.
 //   Digit pairs with i + j > 6 lie below 2^-56 of the largest product and are left
 //   out, as FP64 would round them off.
 // - Per chunk the D_d are joined in 64-bit integers (sum d <= 5 of
@@ -26,9 +27,9 @@
 // - A tile whose chunk scales leave a safe exponent range (infinities, NaN,
 //   magnitudes beyond 2^+-440) is recomputed in FP64 by its epilogue warps.
 //
-// A CTA owns 128 rows x 32 columns. Warps 0-7 find the scales (a first read of
+// A CTA owns 128 rows x 32 columns. Warps 0-15 find the scales (a first read of
 // the chunk's A, which also brings it into L2), sum the orbits and write the digits;
-// one thread issues the matrix instructions; warps 8-11 join the sums; one warp
+// one thread issues the matrix instructions; warps 16-19 join the sums; one warp
 // finds the chunks' tuples. Digit i of A meets digits 0..6-i of W, which lie
 // side by side as one N = 32 (7 - i) operand, so each digit of A is read once from
 // shared memory per step and its products land in the accumulators i..6: 7
@@ -43,16 +44,22 @@ namespace ss {
 
 constexpr int KT_ROWS = 128, KT_COLS = 32, KT_ND = 7;
 constexpr int KT_UNIT = 24;                       // tuples of a unit: 24 / m orbits of one pattern
-constexpr int KT_UPC = 6;                         // units of a chunk
-constexpr int KT_CHUNK = KT_UNIT * KT_UPC;        // 144 tuples
-constexpr int KT_PROD = 256;                      // producer threads: two per row
+constexpr int KT_UPC = 8;                         // units of a chunk: four stages of two
+constexpr int KT_CHUNK = KT_UNIT * KT_UPC;        // 192 tuples
+constexpr int KT_PROD = 512;                      // producer threads: four per row, two groups taking stages in turn
 constexpr int KT_THREADS = KT_PROD + 128 + 64;    // + epilogue + (matrix, table) warps
 // operand layout (K-major, no swizzle): 8 tuples x 8 rows as 128 contiguous bytes
 constexpr int KT_AKG = KT_ROWS * 16;              // bytes of 8 tuples of one digit of A
 constexpr int KT_AD = 6 * KT_AKG;                 // bytes of one digit of A: a stage's two units
 constexpr int KT_WKG = KT_ND * KT_COLS * 16;      // bytes of 8 tuples of all digits of W
-constexpr int KT_STAGE = KT_ND * KT_AD + 6 * KT_WKG;
+constexpr int KT_WST = 6 * KT_WKG;                // bytes of a stage of W
+constexpr int KT_STAGE = KT_ND * KT_AD + KT_WST;
 constexpr unsigned KT_ELO = (1023u - 440u) << 20, KT_EHI = (1023u + 440u) << 20;
+
+template <int N>
+struct KtInt {
+  static constexpr int value = N;
+};
 
 struct KtArgs {
   const double* W;
@@ -62,21 +69,26 @@ struct KtArgs {
   int ytiles;
   int nchunk;
   int upre[9];         // unit prefix per pattern
-  int bits;            // |A| < 2^bits on its grid
+  int bits, up;        // |A| < 2^bits: rounded to 2^(bits - up) and shifted up
   int sh0;             // exponent of a joined sum's unit, less the two scales' exponents
   int opow[4];
+  // prepared by kt_prep_kernel in the call's workspace
+  unsigned char* wdig;  // digits of W by column tile, chunk and stage
+  unsigned* wexp;       // [column tile][chunk][32] scales; top bit: out of range
+  int* tix;             // [chunk][192] tuple indices
+  int* pat;             // [chunk][8] unit patterns, -1: none
 };
 
 struct KtShared {
-  unsigned rowmax[2][KT_ROWS];
+  unsigned short rowmax[4][4][KT_ROWS];  // by chunk mod 4 and quarter: exponent of the largest |A|
   // chunk scales by chunk mod 8: producers run at most two chunks ahead of the
   // matrix warp, and that at most two ahead of the epilogue
   unsigned rowexp[8][KT_ROWS];   // exponent fields
-  unsigned colmax[8][KT_COLS];   // high words of the largest |W|
-  int tix[2][KT_CHUNK];          // tuple indices of a chunk, -1: none
-  int pat[2][KT_UPC];            // pattern of each unit, -1: none
+  unsigned colexp[16][KT_COLS];  // W's, by chunk mod 16 (the table warp runs ahead of the producers)
+  alignas(16) int tix[3][KT_CHUNK];  // tuple indices of a chunk (no tuple left: 0, and W's digits are 0)
+  int pat[3][KT_UPC];            // pattern of each unit, -1: none
   int bad[8];                    // by tile mod 8: a scale is out of range
-  uint64_t tab_full[2], tab_empty[2], st_full[2], st_empty[2], acc_full[2], acc_empty[2], drain;
+  uint64_t tab_full[3], tab_empty[3], mx_full[2], st_full[2], st_empty[2], acc_full[2], acc_empty[2], drain;
   uint32_t tmem;
 };
 
@@ -99,6 +111,11 @@ __device__ __forceinline__ void kt_ld8(uint32_t addr, uint32_t (&r)[8]) {
                : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
                : "r"(addr));
 }
+__device__ __forceinline__ void kt_st8(uint32_t addr, const uint32_t (&r)[8]) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"r"(addr), "r"(r[0]),
+               "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7])
+               : "memory");
+}
 // barrier `id` over n threads; true if `ok` holds in all of them (threads whose
 // bounded wait ran out leave together with the others)
 template <int ID, int N>
@@ -113,14 +130,15 @@ __device__ __forceinline__ bool kt_sync(bool ok) {
   return r != 0;
 }
 
-// |x| on the grid of the scale: 2^(bits) mantissa positions below the scale's
-// next power of two, truncated; signed
-__device__ __forceinline__ long long kt_fixed(double x, unsigned base, int up) {
-  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
-  const unsigned k = (base - (hi & 0x7FFFFFFFu)) >> 20;
-  const unsigned long long mant = (((unsigned long long)((hi & 0x000FFFFFu) | 0x00100000u) << 32) | lo) << up;
-  const long long q = (long long)shr64(mant, k);
-  return (int)hi < 0 ? -q : q;
+// x rounded to the grid of a scale, as two limbs l1 2^24 + l0 of the integer shifted up
+// by `up`: one FP64 addition of 1.5 * 2^52 grid units (high word `magic`) leaves the
+// integer in the low bits (integer shifts of the mantissa took 16 instructions, and this
+// kernel's FP64 pipe is otherwise idle)
+__device__ __forceinline__ void kt_limbs(double x, unsigned magic, int up, int& l0, int& l1) {
+  const double m = __dadd_rn(x, __hiloint2double((int)magic, 0));
+  const unsigned lo = (unsigned)__double2loint(m), hi = (unsigned)__double2hiint(m) - magic;
+  l0 = (int)((lo << up) & 0xFFFFFFu);
+  l1 = (int)__funnelshift_r(lo, hi, 24 - up);
 }
 
 // limbs y1 2^24 + y0 -> the biased digits: byte 3..0 of z1, then byte 2..0 of z0, each digit + 128
@@ -152,26 +170,68 @@ __device__ __forceinline__ void kt_store8(unsigned char* dst, int stride, const 
   *reinterpret_cast<uint4*>(dst + 6 * stride) = kt_pack<0>(z0);
 }
 
+// N tuples' elements of one row (rows past the end read the last one: As)
+template <int N>
+__device__ __forceinline__ void kt_load(const double* As, int64_t S, const int* tix, double* x) {
+  static_assert(N % 4 == 0, "whole int4");
+#pragma unroll
+  for (int e = 0; e < N; e += 4) {
+    const int4 t = *reinterpret_cast<const int4*>(tix + e);
+    x[e] = As[(int64_t)t.x * S];
+    x[e + 1] = As[(int64_t)t.y * S];
+    x[e + 2] = As[(int64_t)t.z * S];
+    x[e + 3] = As[(int64_t)t.w * S];
+  }
+}
+
 // one unit (24 tuples of pattern P) of one row: loads, orbit operator, digits
 template <int D, int P>
-__device__ __forceinline__ void kt_unit(const KParams& kp, const KtArgs& ka, const double* As, bool act, const int* tix,
-                                        unsigned base, unsigned char* dst) {
+__device__ __forceinline__ void kt_unit(const KParams& kp, const KtArgs& ka, const double* As, const int* tix,
+                                        unsigned magic, unsigned char* dst) {
   constexpr int M = Pat<D, P>::M, NO = KT_UNIT / M;
-  double x[KT_UNIT];
+  if constexpr (M == 24) {
+    // one 24-member orbit, by eights of outputs (registers)
+    double x[KT_UNIT];
+    kt_load<KT_UNIT>(As, kp.S, tix, x);
+    int l0[M], l1[M];
 #pragma unroll
-  for (int e = 0; e < KT_UNIT; e++) {
-    const int t = tix[e];
-    x[e] = act && t >= 0 ? As[(int64_t)t * kp.S] : 0.0;
+    for (int v = 0; v < M; v++) {
+      kt_limbs(x[v], magic, ka.up, l0[v], l1[v]);
+    }
+#pragma unroll
+    for (int g = 0; g < 3; g++) {
+      int y0[8], y1[8];
+      unsigned z0[8], z1[8];
+#pragma unroll
+      for (int j = 0; j < 8; j++) { y0[j] = 0; y1[j] = 0; }
+#pragma unroll
+      for (int s = 0; s < fact(D); s++) {
+        const int c = kp.ci[0][s];
+        if (c != 0) {
+#pragma unroll
+          for (int j = 0; j < 8; j++) {
+            y0[j] += c * l0[Pat<D, P>::idx(8 * g + j, s)];
+            y1[j] += c * l1[Pat<D, P>::idx(8 * g + j, s)];
+          }
+        }
+      }
+#pragma unroll
+      for (int j = 0; j < 8; j++) kt_digits(y0[j], y1[j], z0[j], z1[j]);
+      kt_store8(dst + g * KT_AKG, KT_AD, z0, z1);
+    }
+    return;
   }
+  // two batches of twelve tuples (registers)
+  constexpr int NB = 12;
+  double x[NB];
   unsigned z0[KT_UNIT], z1[KT_UNIT];
 #pragma unroll
   for (int o = 0; o < NO; o++) {
+    if (o * M % NB == 0) kt_load<NB>(As, kp.S, tix + o * M, x);
     int l0[M], l1[M], y0[M], y1[M];
 #pragma unroll
     for (int v = 0; v < M; v++) {
-      const long long X = kt_fixed(x[o * M + v], base, 0);
-      l0[v] = (int)((unsigned)X & 0xFFFFFFu);
-      l1[v] = (int)(X >> 24);
+      kt_limbs(x[o * M % NB + v], magic, ka.up, l0[v], l1[v]);
     }
     if constexpr (P == 0) {
 #pragma unroll
@@ -214,23 +274,24 @@ __device__ __forceinline__ void kt_unit(const KParams& kp, const KtArgs& ka, con
     }
 #pragma unroll
     for (int u = 0; u < M; u++) kt_digits(y0[u], y1[u], z0[o * M + u], z1[o * M + u]);
-  }
 #pragma unroll
-  for (int g = 0; g < 3; g++) kt_store8(dst + g * KT_AKG, KT_AD, z0 + 8 * g, z1 + 8 * g);
+    for (int g = 0; g < 3; g++)  // eights that this orbit completed
+      if (o * M < 8 * g + 8 && (o + 1) * M >= 8 * g + 8) kt_store8(dst + g * KT_AKG, KT_AD, z0 + 8 * g, z1 + 8 * g);
+  }
 }
 
 template <int D>
-__device__ __forceinline__ void kt_unit_any(const KParams& kp, const KtArgs& ka, int p, const double* As, bool act,
-                                            const int* tix, unsigned base, unsigned char* dst) {
+__device__ __forceinline__ void kt_unit_any(const KParams& kp, const KtArgs& ka, int p, const double* As,
+                                            const int* tix, unsigned magic, unsigned char* dst) {
   switch (p) {
-    case 0: kt_unit<D, 0>(kp, ka, As, act, tix, base, dst); break;
-    case 1: kt_unit<D, 1>(kp, ka, As, act, tix, base, dst); break;
-    case 2: if constexpr (npatterns(D) > 2) kt_unit<D, 2>(kp, ka, As, act, tix, base, dst); break;
-    case 3: if constexpr (npatterns(D) > 3) kt_unit<D, 3>(kp, ka, As, act, tix, base, dst); break;
-    case 4: if constexpr (npatterns(D) > 4) kt_unit<D, 4>(kp, ka, As, act, tix, base, dst); break;
-    case 5: if constexpr (npatterns(D) > 4) kt_unit<D, 5>(kp, ka, As, act, tix, base, dst); break;
-    case 6: if constexpr (npatterns(D) > 4) kt_unit<D, 6>(kp, ka, As, act, tix, base, dst); break;
-    case 7: if constexpr (npatterns(D) > 4) kt_unit<D, 7>(kp, ka, As, act, tix, base, dst); break;
+    case 0: kt_unit<D, 0>(kp, ka, As, tix, magic, dst); break;
+    case 1: kt_unit<D, 1>(kp, ka, As, tix, magic, dst); break;
+    case 2: if constexpr (npatterns(D) > 2) kt_unit<D, 2>(kp, ka, As, tix, magic, dst); break;
+    case 3: if constexpr (npatterns(D) > 3) kt_unit<D, 3>(kp, ka, As, tix, magic, dst); break;
+    case 4: if constexpr (npatterns(D) > 4) kt_unit<D, 4>(kp, ka, As, tix, magic, dst); break;
+    case 5: if constexpr (npatterns(D) > 4) kt_unit<D, 5>(kp, ka, As, tix, magic, dst); break;
+    case 6: if constexpr (npatterns(D) > 4) kt_unit<D, 6>(kp, ka, As, tix, magic, dst); break;
+    case 7: if constexpr (npatterns(D) > 4) kt_unit<D, 7>(kp, ka, As, tix, magic, dst); break;
     default:  // no tuples left: digits of zero
       const unsigned z[8] = {0x80808080u, 0x80808080u, 0x80808080u, 0x80808080u, 0x80808080u, 0x80808080u, 0x80808080u, 0x80808080u};
       for (int g = 0; g < 3; g++) kt_store8(dst + g * KT_AKG, KT_AD, z, z);
@@ -239,7 +300,7 @@ __device__ __forceinline__ void kt_unit_any(const KParams& kp, const KtArgs& ka,
 
 // the orbit `rank` of pattern P into its unit's entries tix[0..m)
 template <int D, int P>
-__device__ __forceinline__ void kt_orbit(const KParams& kp, const KtArgs& ka, int64_t rank, int* tix) {
+__device__ __forceinline__ void kt_orbit(const KParams& kp, const KtArgs& ka, int64_t rank, int* tix, signed char* none) {
   constexpr int M = Pat<D, P>::M;
   int v[4] = {0, 0, 0, 0};
   const bool ok = rank < kp.norb[P];
@@ -249,7 +310,8 @@ __device__ __forceinline__ void kt_orbit(const KParams& kp, const KtArgs& ka, in
     int t = 0;
 #pragma unroll
     for (int k = 0; k < D; k++) t += v[Pat<D, P>::lab(u, k)] * ka.opow[k];
-    tix[u] = ok ? t : -1;
+    tix[u] = t;
+    none[u] = ok ? 0 : -1;
   }
 }
 
@@ -259,6 +321,85 @@ __device__ __forceinline__ int kt_members(int p) {
   if constexpr (D == 2) return p == 0 ? 2 : 1;
   else if constexpr (D == 3) return p == 0 ? 6 : (p == 3 ? 1 : 3);
   else return p == 0 ? 24 : (p <= 3 ? 12 : (p == 4 ? 6 : (p == 7 ? 1 : 4)));
+}
+
+// W once per call: a CTA takes a chunk and 32 columns, finds the chunk's tuples (kept for
+// the main kernel), the columns' scales and the digits, in the layout of a stage.
+// (Digitised by every row tile's CTA instead, W cost 0.16 of 0.56 ms on A[48^3,8^3].)
+template <int D>
+__global__ void __launch_bounds__(256) kt_prep_kernel(const __grid_constant__ KParams kp, const __grid_constant__ KtArgs ka) {
+  __shared__ int tix[KT_CHUNK];
+  __shared__ signed char none[KT_CHUNK];
+  __shared__ unsigned colmax[KT_COLS];
+  const int tid = threadIdx.x, ch = blockIdx.x, yt = blockIdx.y;
+  const int nunit = ka.upre[npatterns(D)];
+  if (tid < KT_COLS) colmax[tid] = 0;
+  if (tid < KT_CHUNK) {
+    tix[tid] = 0;
+    none[tid] = -1;
+  }
+  __syncthreads();
+  if (tid < KT_CHUNK) {
+    // thread o + 24 u: orbit o of unit u
+    const int u = tid / KT_UNIT, o = tid % KT_UNIT, g = ch * KT_UPC + u;
+    int p = -1;
+    if (g < nunit) {
+      p = 0;
+#pragma unroll
+      for (int r = 1; r < npatterns(D); r++)
+        if (g >= ka.upre[r]) p = r;
+      const int m = kt_members<D>(p), no = KT_UNIT / m;
+      if (o < no) {
+        const int64_t rank = (int64_t)(g - ka.upre[p]) * no + o;
+        int* dst = tix + u * KT_UNIT + o * m;
+        signed char* dn = none + u * KT_UNIT + o * m;
+        switch (p) {
+          case 0: kt_orbit<D, 0>(kp, ka, rank, dst, dn); break;
+          case 1: kt_orbit<D, 1>(kp, ka, rank, dst, dn); break;
+          case 2: if constexpr (npatterns(D) > 2) kt_orbit<D, 2>(kp, ka, rank, dst, dn); break;
+          case 3: if constexpr (npatterns(D) > 3) kt_orbit<D, 3>(kp, ka, rank, dst, dn); break;
+          case 4: if constexpr (npatterns(D) > 4) kt_orbit<D, 4>(kp, ka, rank, dst, dn); break;
+          case 5: if constexpr (npatterns(D) > 4) kt_orbit<D, 5>(kp, ka, rank, dst, dn); break;
+          case 6: if constexpr (npatterns(D) > 4) kt_orbit<D, 6>(kp, ka, rank, dst, dn); break;
+          case 7: if constexpr (npatterns(D) > 4) kt_orbit<D, 7>(kp, ka, rank, dst, dn); break;
+        }
+      }
+    }
+    if (yt == 0 && o == 0) ka.pat[ch * KT_UPC + u] = p;
+  }
+  __syncthreads();
+  if (yt == 0 && tid < KT_CHUNK) ka.tix[ch * KT_CHUNK + tid] = tix[tid];
+  const int y = tid & 31, q = tid >> 5;
+  const bool act = (int64_t)yt * KT_COLS + y < ka.Y;
+  const double* Wy = ka.W + (int64_t)yt * KT_COLS + y;
+  auto load = [&](int e) { return act && none[e] == 0 ? Wy[(int64_t)tix[e] * ka.ldw] : 0.0; };
+  unsigned m = 0;
+  for (int e = q; e < KT_CHUNK; e += 8) {
+    const double v = load(e);
+    m = max(m, ((unsigned)__double2hiint(v) & 0x7FFFFFFFu) | ((unsigned)__double2loint(v) != 0));
+  }
+  atomicMax(&colmax[y], m);
+  __syncthreads();
+  m = colmax[y];
+  unsigned E = m & 0x7FF00000u, bad = 0;
+  if (E < KT_ELO || E > KT_EHI) {
+    bad = m != 0 ? 0x80000000u : 0;
+    E = KT_ELO;
+  }
+  if (q == 0) ka.wexp[((int64_t)yt * ka.nchunk + ch) * KT_COLS + y] = E | bad;
+  // largest |W| below 2^51, then shifted up by 3
+  const unsigned magic = (E + (2u << 20)) | 0x80000u;
+  for (int kg = q; kg < KT_CHUNK / 8; kg += 8) {
+    unsigned z0[8], z1[8];
+#pragma unroll
+    for (int e = 0; e < 8; e++) {
+      int l0, l1;
+      kt_limbs(load(kg * 8 + e), magic, 3, l0, l1);
+      kt_digits(l0, l1, z0[e], z1[e]);
+    }
+    unsigned char* dst = ka.wdig + (((int64_t)yt * ka.nchunk + ch) * 4 + kg / 6) * KT_WST + kg % 6 * KT_WKG + y * 16;
+    kt_store8(dst, KT_COLS * 16, z0, z1);
+  }
 }
 
 // FP64 form of one tile (rare): a thread per row, KC's loop over the orbits
@@ -302,10 +443,13 @@ __global__ void __launch_bounds__(KT_THREADS, 1) kt_kernel(const __grid_constant
   __shared__ KtShared sh;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   if (tid == 0) {
-    for (int i = 0; i < 2; i++) {
+    for (int i = 0; i < 3; i++) {
       mbar_init(&sh.tab_full[i], 32);
       mbar_init(&sh.tab_empty[i], KT_PROD);
-      mbar_init(&sh.st_full[i], KT_PROD);
+    }
+    for (int i = 0; i < 2; i++) {
+      mbar_init(&sh.mx_full[i], KT_PROD);
+      mbar_init(&sh.st_full[i], KT_PROD / 2 + 1);  // a group, and W's copy
       mbar_init(&sh.st_empty[i], 1);
       mbar_init(&sh.acc_full[i], 1);
       mbar_init(&sh.acc_empty[i], 128);
@@ -313,10 +457,9 @@ __global__ void __launch_bounds__(KT_THREADS, 1) kt_kernel(const __grid_constant
     mbar_init(&sh.drain, 1);
     fence_mbar_init();
   }
-  if (tid < KT_COLS)
-    for (int i = 0; i < 8; i++) sh.colmax[i][tid] = 0;
   if (tid < 8) sh.bad[tid] = 0;
-  if (warp == 12) {
+  constexpr int MMA_WARP = KT_PROD / 32 + 4;
+  if (warp == MMA_WARP) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_u32(&sh.tmem)) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   }
@@ -329,98 +472,81 @@ __global__ void __launch_bounds__(KT_THREADS, 1) kt_kernel(const __grid_constant
   const long long lim = kp.wait_limit;
   bool ok = true;  // every wait is bounded: a role whose wait runs out reports and leaves its loop
 
-  if (warp < 8) {
+  if (warp < KT_PROD / 32) {
     // ---- producers: scales, orbit sums, digits ----
-    const int row = tid & (KT_ROWS - 1), half = tid >> 7;
-    int c = 0, n = 0, it = 0;  // chunks, stages and tiles so far
-    for (int64_t tile = blockIdx.x; tile < ka.tiles; tile += gridDim.x, it++) {
-      const int64_t s = tile / ka.ytiles * KT_ROWS + row, y0 = tile % ka.ytiles * KT_COLS;
-      const int ny = (int)min((int64_t)KT_COLS, ka.Y - y0);
-      const bool act = s < kp.S;
-      const double* As = static_cast<const double*>(kp.A) + s;
-      const double* Wy = ka.W + y0 + (tid & 31);
-      const bool wact = (tid & 31) < ny;
-      for (int ch = 0; ch < ka.nchunk; ch++, c++) {
-        const int* tix = sh.tix[c & 1];
-        ok = kt_sync<1, KT_PROD>(ok && mbar_wait(&sh.tab_full[c & 1], (c >> 1) & 1, lim));
-        if (!ok) break;
-        // scales: the largest |A| of the row and |W| of the column in this chunk
-        unsigned mx = 0, low = 0, wmx = 0, wlow = 0;
+    const int row = tid & (KT_ROWS - 1), quarter = tid >> 7, half = quarter & 1, group = tid >> 8;
+    const int64_t step = gridDim.x;
+    auto row_of = [&](int64_t tile) {
+      const int64_t s = tile / ka.ytiles * KT_ROWS + row;
+      return static_cast<const double*>(kp.A) + (s < kp.S ? s : kp.S - 1);
+    };
+    // the largest |A| of the row in chunk c of a tile (a quarter of the tuples per
+    // thread); run one chunk ahead, so that its loads and the meeting of all producers
+    // hide under the chunk before
+    auto maxima = [&](int64_t tile, int c) {
+      if (!mbar_wait(&sh.tab_full[c % 3], (c / 3) & 1, lim)) return false;
+      const int* tix = sh.tix[c % 3];
+      const double* As = row_of(tile);
+      unsigned mx = 0;
 #pragma unroll 1
-        for (int j = 0; j < 3; j++) {
-          const int* te = tix + (2 * j + half) * KT_UNIT;
-          double v[KT_UNIT];
+      for (int j = 0; j < 3; j++) {
+        constexpr int N = KT_CHUNK / 12;
+        double v[N];
+        kt_load<N>(As, kp.S, tix + quarter * (KT_CHUNK / 4) + j * N, v);
+        unsigned m = 0;
 #pragma unroll
-          for (int e = 0; e < KT_UNIT; e++) {
-            const int t = te[e];
-            v[e] = act && t >= 0 ? As[(int64_t)t * kp.S] : 0.0;
-          }
+        for (int e = 0; e < N; e++) m = max(m, (unsigned)__double2hiint(v[e]) & 0x7FFFFFFFu);
+        if (m == 0) {  // zeros, or magnitudes below 2^-1042: the latter are out of range
 #pragma unroll
-          for (int e = 0; e < KT_UNIT; e++) {
-            mx = max(mx, (unsigned)__double2hiint(v[e]) & 0x7FFFFFFFu);
-            low |= (unsigned)__double2loint(v[e]);
-          }
+          for (int e = 0; e < N; e++) m |= (unsigned)__double2loint(v[e]) != 0;
         }
-#pragma unroll
-        for (int j = 0; j < KT_CHUNK / 8; j++) {
-          const int t = tix[(tid >> 5) + 8 * j];
-          const double v = wact && t >= 0 ? Wy[(int64_t)t * ka.ldw] : 0.0;
-          wmx = max(wmx, (unsigned)__double2hiint(v) & 0x7FFFFFFFu);
-          wlow |= (unsigned)__double2loint(v);
+        mx = max(mx, m);
+      }
+      // exponents only; 1 (out of range) for subnormal maxima
+      sh.rowmax[c & 3][quarter][row] = (unsigned short)(mx >> 20 == 0 && mx != 0 ? 1 : mx >> 20);
+      mbar_arrive(&sh.mx_full[c & 1]);
+      return true;
+    };
+    int c = 0, n = 0, it = 0;  // chunks, stages and tiles so far
+    if (blockIdx.x < ka.tiles) ok = maxima(blockIdx.x, 0);
+    for (int64_t tile = blockIdx.x; ok && tile < ka.tiles; tile += step, it++) {
+      const double* As = row_of(tile);
+      const unsigned char* wd = ka.wdig + tile % ka.ytiles * ka.nchunk * 4 * KT_WST;
+      for (int ch = 0; ok && ch < ka.nchunk; ch++, c++) {
+        const int64_t nt = ch + 1 < ka.nchunk ? tile : tile + step;
+        if (nt < ka.tiles) ok = maxima(nt, c + 1);
+        ok = ok && mbar_wait(&sh.mx_full[c & 1], (c >> 1) & 1, lim);
+        if (!ok) break;
+        const int* tix = sh.tix[c % 3];
+        const unsigned short* rm = &sh.rowmax[c & 3][0][row];
+        unsigned E = max(max(rm[0], rm[KT_ROWS]), max(rm[2 * KT_ROWS], rm[3 * KT_ROWS])) << 20;
+        if (E < KT_ELO || E > KT_EHI) {
+          if (E != 0) sh.bad[it & 7] = 1;
+          E = KT_ELO;
         }
-        if (wmx == 0 && wlow != 0) wmx = 1;  // subnormal only: out of range below
-        if (mx == 0 && low != 0) mx = 1;
-        sh.rowmax[half][row] = mx;
-        atomicMax(&sh.colmax[c & 7][tid & 31], wmx);
-        kt_sync<1, KT_PROD>(true);
-        mx = max(sh.rowmax[0][row], sh.rowmax[1][row]);
-        wmx = sh.colmax[c & 7][tid & 31];
-        auto scale = [&](unsigned m) {
-          unsigned E = m & 0x7FF00000u;
-          if (E < KT_ELO || E > KT_EHI) {
-            if (m != 0) sh.bad[it & 7] = 1;
-            E = KT_ELO;
-          }
-          return E;
-        };
-        const unsigned E = scale(mx), Ew = scale(wmx);
-        if (half == 0) sh.rowexp[c & 7][row] = E;
-        if (tid < 32) sh.colmax[(c + 2) & 7][tid] = 0;  // of chunk c - 6
-        // largest |A| below 2^bits, largest |W| below 2^54
-        const unsigned base = (E | 0xFFFFFu) + ((unsigned)(53 - ka.bits) << 20);
-        const unsigned wbase = Ew | 0xFFFFFu;
+        if (tid < 32 && sh.colexp[c & 15][tid] >> 31) sh.bad[it & 7] = 1;
+        if (quarter == 0) sh.rowexp[c & 7][row] = E;
+        // largest |A| below 2^(bits - up)
+        const unsigned magic = (E + ((unsigned)(53 - ka.bits + ka.up) << 20)) | 0x80000u;
         const int ns = stages_of(ch);
         for (int j = 0; ok && j < ns; j++, n++) {
+          if ((n & 1) != group) continue;  // the other group's stage
           unsigned char* st = kt_smem + (n & 1) * KT_STAGE;
           ok = mbar_wait(&sh.st_empty[n & 1], ((n >> 1) & 1) ^ 1, lim);
-          if (!ok) break;  // all leave at the next chunk's barrier
-          const int u = 2 * j + half;
-          kt_unit_any<D>(kp, ka, sh.pat[c & 1][u], As, act, tix + u * KT_UNIT, base,
-                         st + half * 3 * KT_AKG + row * 16);
-          if (tid < 6 * 32) {
-            const int kg = tid >> 5;
-            unsigned z0[8], z1[8];
-            double w[8];
-#pragma unroll
-            for (int e = 0; e < 8; e++) {
-              const int t = tix[2 * j * KT_UNIT + kg * 8 + e];
-              w[e] = wact && t >= 0 ? Wy[(int64_t)t * ka.ldw] : 0.0;
-            }
-#pragma unroll
-            for (int e = 0; e < 8; e++) {
-              const long long X = kt_fixed(w[e], wbase, 1);
-              kt_digits((int)((unsigned)X & 0xFFFFFFu), (int)(X >> 24), z0[e], z1[e]);
-            }
-            kt_store8(st + KT_ND * KT_AD + kg * KT_WKG + (tid & 31) * 16, KT_COLS * 16, z0, z1);
+          if (!ok) break;
+          if ((tid & 255) == 0) {
+            mbar_arrive_expect_tx(&sh.st_full[n & 1], KT_WST);
+            bulk_g2s(st + KT_ND * KT_AD, wd + ((int64_t)ch * 4 + j) * KT_WST, KT_WST, &sh.st_full[n & 1]);
           }
+          const int u = 2 * j + half;
+          kt_unit_any<D>(kp, ka, sh.pat[c % 3][u], As, tix + u * KT_UNIT, magic, st + half * 3 * KT_AKG + row * 16);
           kt_proxy_fence();
           mbar_arrive(&sh.st_full[n & 1]);
         }
-        mbar_arrive(&sh.tab_empty[c & 1]);
+        mbar_arrive(&sh.tab_empty[c % 3]);
       }
-      if (!kt_sync<1, KT_PROD>(ok)) { ok = false; break; }
     }
-  } else if (warp < 12) {
+  } else if (warp < MMA_WARP) {
     // ---- epilogue: join the digit sums of a chunk, add up the chunks ----
     const int row = tid - KT_PROD;
     const uint32_t lanes = (uint32_t)(warp & 3) << 21;  // TMEM lane 32 (warp mod 4)
@@ -428,50 +554,63 @@ __global__ void __launch_bounds__(KT_THREADS, 1) kt_kernel(const __grid_constant
     for (int64_t tile = blockIdx.x; ok && tile < ka.tiles; tile += gridDim.x, it++) {
       const int64_t s = tile / ka.ytiles * KT_ROWS + row, y0 = tile % ka.ytiles * KT_COLS;
       const int ny = (int)min((int64_t)KT_COLS, ka.Y - y0);
-      double acc[KT_COLS];
-#pragma unroll
-      for (int y = 0; y < KT_COLS; y++) acc[y] = 0.0;
+      bool bad = false;
       for (int ch = 0; ch < ka.nchunk; ch++, c++) {
         ok = __all_sync(0xffffffffu, mbar_wait(&sh.acc_full[c & 1], (c >> 1) & 1, lim));
         if (!ok) break;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        const bool last = ch == ka.nchunk - 1;
+        if (last) bad = sh.bad[it & 7] != 0;  // every scale of the tile is known
         const int er = (int)(sh.rowexp[c & 7][row] >> 20) + ka.sh0;
         const uint32_t t0 = tmem + (uint32_t)(c & 1) * 256 + lanes;
-#pragma unroll
+        // the FP64 sums of the 32 columns live in the 2 x 32 accumulator columns that the
+        // digit sums leave free (in registers they would cap the producers' share)
+        const uint32_t tlo = tmem + lanes + KT_ND * KT_COLS, thi = tlo + 256;
+#pragma unroll 1
         for (int yb = 0; yb < KT_COLS; yb += 8) {
-          uint32_t d[KT_ND][8];
+          uint32_t d[KT_ND][8], lo[8] = {}, hi[8] = {};
 #pragma unroll
           for (int i = 0; i < KT_ND; i++) kt_ld8(t0 + i * KT_COLS + yb, d[i]);
+          if (ch > 0) {
+            kt_ld8(tlo + yb, lo);
+            kt_ld8(thi + yb, hi);
+          }
           asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
           for (int y = 0; y < 8; y++) {
             int v[KT_ND];
 #pragma unroll
             for (int i = 0; i < KT_ND; i++) v[i] = __float2int_rn(__uint_as_float(d[i][y]));
-            // |D_0| <= 2^20.2, |D_1| <= 2^22.2, |D_d| < 2^24: the joined sum stays below 2^61
+            // |D_0| <= 2^19.6, |D_d| <= 192 d 2^14: the joined sum stays below 2^61
             long long V = (long long)((unsigned long long)(unsigned)(v[0] * 256 + v[1]) << 32);
             V += (long long)v[2] * (1 << 24) + (long long)v[3] * (1 << 16);
             V += (long long)v[4] * 256 + (long long)(v[5] + ((v[6] + 128) >> 8));
-            acc[yb + y] += kt_to_double(V, er + (int)(max(sh.colmax[c & 7][yb + y], KT_ELO) >> 20));
+            const double a = __hiloint2double((int)hi[y], (int)lo[y]) +
+                             kt_to_double(V, er + (int)((sh.colexp[c & 15][yb + y] & 0x7FF00000u) >> 20));
+            lo[y] = (unsigned)__double2loint(a);
+            hi[y] = (unsigned)__double2hiint(a);
+          }
+          if (!last) {
+            kt_st8(tlo + yb, lo);
+            kt_st8(thi + yb, hi);
+          } else if (!bad && s < kp.S) {
+#pragma unroll
+            for (int y = 0; y < 8; y++)
+              if (yb + y < ny) ka.C[s + ka.ldc * (y0 + yb + y)] = __hiloint2double((int)hi[y], (int)lo[y]);
           }
         }
+        asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         mbar_arrive(&sh.acc_empty[c & 1]);
       }
       ok = kt_sync<2, 128>(ok);
       if (!ok) break;
-      const int bad = sh.bad[it & 7];
-      kt_sync<2, 128>(true);
       if (bad) {
         if (row == 0) sh.bad[it & 7] = 0;
         kt_tile_fp64<D>(kp, ka, s, y0, ny);
-      } else if (s < kp.S) {
-#pragma unroll
-        for (int y = 0; y < KT_COLS; y++)
-          if (y < ny) ka.C[s + ka.ldc * (y0 + y)] = acc[y];
       }
     }
-  } else if (warp == 12) {
+  } else if (warp == MMA_WARP) {
     // ---- matrix instructions, by one thread ----
     if (lane == 0) {
       const uint32_t sbase = smem_u32(kt_smem);
@@ -503,60 +642,59 @@ __global__ void __launch_bounds__(KT_THREADS, 1) kt_kernel(const __grid_constant
       ok = mbar_wait(&sh.drain, 0, lim) && ok;
     }
     __syncwarp();
-  } else {
-    // ---- the chunks' tuples ----
+  } else if (warp == MMA_WARP + 1) {
+    // ---- the chunks' tuples and W's scales, ahead of the producers ----
     int c = 0;
     for (int64_t tile = blockIdx.x; ok && tile < ka.tiles; tile += gridDim.x)
       for (int ch = 0; ok && ch < ka.nchunk; ch++, c++) {
-        if (!mbar_wait(&sh.tab_empty[c & 1], ((c >> 1) & 1) ^ 1, lim)) { ok = false; break; }
-        int p[KT_UPC], mo = 1;
-#pragma unroll
-        for (int u = 0; u < KT_UPC; u++) {
-          const int g = ch * KT_UPC + u;
-          p[u] = -1;
-          if (g < nunit) {
-            p[u] = 0;
-#pragma unroll
-            for (int q = 1; q < npatterns(D); q++)
-              if (g >= ka.upre[q]) p[u] = q;
-            mo = max(mo, KT_UNIT / kt_members<D>(p[u]));
-          }
-          if (lane == 0) sh.pat[c & 1][u] = p[u];
+        if (!mbar_wait(&sh.tab_empty[c % 3], ((c / 3) & 1) ^ 1, lim)) { ok = false; break; }
+        const int64_t s0 = tile / ka.ytiles * KT_ROWS;
+        const unsigned bytes = (unsigned)(min((int64_t)KT_ROWS, kp.S - s0) * 8) & ~15u;
+        for (int e = lane; e < KT_CHUNK; e += 32) {
+          const int t = ka.tix[ch * KT_CHUNK + e];
+          sh.tix[c % 3][e] = t;
+          // the tuple's rows of A on their way to L2
+          const double* a = static_cast<const double*>(kp.A) + (int64_t)t * kp.S + s0;
+          if (((uintptr_t)a & 15) == 0 && bytes > 0)
+            asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(a), "r"(bytes) : "memory");
         }
-        for (int q = lane; q < KT_UPC * mo; q += 32) {
-          const int u = q % KT_UPC, o = q / KT_UPC, g = ch * KT_UPC + u;
-          if (g >= nunit) {
-            if (o == 0)
-              for (int e = 0; e < KT_UNIT; e++) sh.tix[c & 1][u * KT_UNIT + e] = -1;
-            continue;
-          }
-          int pp = 0;
-#pragma unroll
-          for (int r = 1; r < npatterns(D); r++)
-            if (g >= ka.upre[r]) pp = r;
-          const int m = kt_members<D>(pp), no = KT_UNIT / m;
-          if (o >= no) continue;
-          const int64_t rank = (int64_t)(g - ka.upre[pp]) * no + o;
-          int* dst = sh.tix[c & 1] + u * KT_UNIT + o * m;
-          switch (pp) {
-            case 0: kt_orbit<D, 0>(kp, ka, rank, dst); break;
-            case 1: kt_orbit<D, 1>(kp, ka, rank, dst); break;
-            case 2: if constexpr (npatterns(D) > 2) kt_orbit<D, 2>(kp, ka, rank, dst); break;
-            case 3: if constexpr (npatterns(D) > 3) kt_orbit<D, 3>(kp, ka, rank, dst); break;
-            case 4: if constexpr (npatterns(D) > 4) kt_orbit<D, 4>(kp, ka, rank, dst); break;
-            case 5: if constexpr (npatterns(D) > 4) kt_orbit<D, 5>(kp, ka, rank, dst); break;
-            case 6: if constexpr (npatterns(D) > 4) kt_orbit<D, 6>(kp, ka, rank, dst); break;
-            case 7: if constexpr (npatterns(D) > 4) kt_orbit<D, 7>(kp, ka, rank, dst); break;
-          }
-        }
-        mbar_arrive(&sh.tab_full[c & 1]);
+        if (lane < KT_UPC) sh.pat[c % 3][lane] = ka.pat[ch * KT_UPC + lane];
+        sh.colexp[c & 15][lane] = ka.wexp[(tile % ka.ytiles * ka.nchunk + ch) * KT_COLS + lane];
+        mbar_arrive(&sh.tab_full[c % 3]);
       }
   }
   if (!ok) report_timeout(kp);
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  if (warp == 12) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem));
+  if (warp == MMA_WARP) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem));
+}
+
+// The library's memory pool for KT's workspaces on a device: freed blocks up to 32 MB
+// stay with it between calls (the default pool would return them to the system at every
+// synchronisation and map them again, milliseconds). Null if the device has no pools.
+inline cudaMemPool_t kt_pool(int dev) {
+  static DeviceCache cache;
+  long long v = 0;
+  const int rc = cache.get(dev, &v, [&](long long* val) {
+    cudaMemPoolProps props{};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.handleTypes = cudaMemHandleTypeNone;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = dev;
+    cudaMemPool_t p = nullptr;
+    cudaError_t err = cudaMemPoolCreate(&p, &props);
+    if (err != cudaSuccess) return (int)err;
+    unsigned long long keep = 32ull << 20;
+    err = cudaMemPoolSetAttribute(p, cudaMemPoolAttrReleaseThreshold, &keep);
+    *val = (long long)(uintptr_t)p;
+    return (int)err;
+  });
+  if (rc != 0) {
+    cudaGetLastError();
+    return nullptr;
+  }
+  return (cudaMemPool_t)(uintptr_t)v;
 }
 
 // Whether KT takes the contraction: exact arithmetic with integer coefficients
@@ -585,7 +723,8 @@ bool launch_kt(const KParams& kp, const double* W, int64_t Y, int64_t ldw, doubl
   ka.ldc = ldc;
   ka.ytiles = (int)((Y + KT_COLS - 1) / KT_COLS);
   ka.tiles = (kp.S + KT_ROWS - 1) / KT_ROWS * ka.ytiles;
-  ka.bits = lg > 0 ? 54 - lg : 53;  // the 53 bits of an FP64 mantissa are enough
+  ka.bits = 54 - lg;
+  ka.up = ka.bits > 51 ? ka.bits - 51 : 0;  // the rounding addition holds 51 bits
   // kp.cexp = (53 - 2 W + kdrop + aexp) << 20 + 0x80000, aexp = the coefficients' scale;
   // a joined sum counts 2^56 of the products' units 2^(E_A + 1 - bits + aexp) 2^(E_W - 53)
   const int aexp = ((kp.cexp - 0x80000) >> 20) - 53 + 2 * kp.W - kp.kdrop;
@@ -620,9 +759,30 @@ bool launch_kt(const KParams& kp, const double* W, int64_t Y, int64_t ldw, doubl
     *e = rc < 0 ? cudaErrorInvalidDevice : (cudaError_t)rc;
     return true;
   }
+  // workspace: the digits, scales and tuples; stream-ordered, so that calls on different
+  // streams and threads have their own and nothing outlives the call
+  const int64_t nd = (int64_t)ka.ytiles * ka.nchunk;
+  const int64_t bw = nd * 4 * KT_WST, be = nd * KT_COLS * 4, bt = (int64_t)ka.nchunk * KT_CHUNK * 4,
+                bp = (int64_t)ka.nchunk * KT_UPC * 4;
+  unsigned char* ws = nullptr;
+  cudaMemPool_t pool = kt_pool(dev);
+  if (!pool || ka.ytiles > 65535 || cudaMallocFromPoolAsync((void**)&ws, (size_t)(bw + be + bt + bp), pool, st) != cudaSuccess) {
+    cudaGetLastError();
+    return false;  // KC needs no workspace
+  }
+  ka.wdig = ws;
+  ka.wexp = reinterpret_cast<unsigned*>(ws + bw);
+  ka.tix = reinterpret_cast<int*>(ws + bw + be);
+  ka.pat = reinterpret_cast<int*>(ws + bw + be + bt);
   const int64_t grid = ka.tiles < sms ? ka.tiles : sms;
-  kt_kernel<D><<<(unsigned)grid, KT_THREADS, 2 * KT_STAGE, st>>>(kp, ka);
+  kt_prep_kernel<D><<<dim3((unsigned)ka.nchunk, (unsigned)ka.ytiles), 256, 0, st>>>(kp, ka);
   *e = cudaGetLastError();
+  if (*e == cudaSuccess) {
+    kt_kernel<D><<<(unsigned)grid, KT_THREADS, 2 * KT_STAGE, st>>>(kp, ka);
+    *e = cudaGetLastError();
+  }
+  const cudaError_t f = cudaFreeAsync(ws, st);
+  if (*e == cudaSuccess) *e = f;
   return true;
 }
 
