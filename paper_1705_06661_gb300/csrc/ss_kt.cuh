@@ -130,15 +130,19 @@ __device__ __forceinline__ bool kt_sync(bool ok) {
   return r != 0;
 }
 
-// x rounded to the grid of a scale, as two limbs l1 2^24 + l0 of the integer shifted up
-// by `up`: one FP64 addition of 1.5 * 2^52 grid units (high word `magic`) leaves the
-// integer in the low bits (integer shifts of the mantissa took 16 instructions, and this
-// kernel's FP64 pipe is otherwise idle)
-__device__ __forceinline__ void kt_limbs(double x, unsigned magic, int up, int& l0, int& l1) {
-  const double m = __dadd_rn(x, __hiloint2double((int)magic, 0));
-  const unsigned lo = (unsigned)__double2loint(m), hi = (unsigned)__double2hiint(m) - magic;
-  l0 = (int)((lo << up) & 0xFFFFFFu);
-  l1 = (int)__funnelshift_r(lo, hi, 24 - up);
+// x on the grid of a scale as two limbs l1 2^24 + l0 of a signed integer, shifted up by
+// `up`: the mantissa shifted right by (base - |x|'s high word) >> 20 places (base: the
+// scale's exponent field, plus the places that the grid drops, with 20 ones below it).
+// (One FP64 addition of 1.5 * 2^52 grid units does the same in five instructions, but at
+// two FP64 operations per SM and clock: 2509 against 2275 us on A[48^3,16^3].)
+__device__ __forceinline__ void kt_limbs(double x, unsigned base, int up, int& l0, int& l1) {
+  const unsigned xh = (unsigned)__double2hiint(x), xl = (unsigned)__double2loint(x);
+  const unsigned k = (base - (xh & 0x7FFFFFFFu)) >> 20;
+  const unsigned long long mant = ((unsigned long long)((xh & 0x000FFFFFu) | 0x00100000u) << 32) | xl;
+  const long long q = (long long)shr64(mant, k);
+  const long long X = (int)xh < 0 ? -q : q;
+  l0 = (int)(((unsigned)X << up) & 0xFFFFFFu);
+  l1 = (int)(X >> (24 - up));
 }
 
 // limbs y1 2^24 + y0 -> the biased digits: byte 3..0 of z1, then byte 2..0 of z0, each digit + 128
@@ -187,7 +191,7 @@ __device__ __forceinline__ void kt_load(const double* As, int64_t S, const int* 
 // one unit (24 tuples of pattern P) of one row: loads, orbit operator, digits
 template <int D, int P>
 __device__ __forceinline__ void kt_unit(const KParams& kp, const KtArgs& ka, const double* As, const int* tix,
-                                        unsigned magic, unsigned char* dst) {
+                                        unsigned base, unsigned char* dst) {
   constexpr int M = Pat<D, P>::M, NO = KT_UNIT / M;
   if constexpr (M == 24) {
     // one 24-member orbit, by eights of outputs (registers)
@@ -196,7 +200,7 @@ __device__ __forceinline__ void kt_unit(const KParams& kp, const KtArgs& ka, con
     int l0[M], l1[M];
 #pragma unroll
     for (int v = 0; v < M; v++) {
-      kt_limbs(x[v], magic, ka.up, l0[v], l1[v]);
+      kt_limbs(x[v], base, ka.up, l0[v], l1[v]);
     }
 #pragma unroll
     for (int g = 0; g < 3; g++) {
@@ -231,7 +235,7 @@ __device__ __forceinline__ void kt_unit(const KParams& kp, const KtArgs& ka, con
     int l0[M], l1[M], y0[M], y1[M];
 #pragma unroll
     for (int v = 0; v < M; v++) {
-      kt_limbs(x[o * M % NB + v], magic, ka.up, l0[v], l1[v]);
+      kt_limbs(x[o * M % NB + v], base, ka.up, l0[v], l1[v]);
     }
     if constexpr (P == 0) {
 #pragma unroll
@@ -282,16 +286,16 @@ __device__ __forceinline__ void kt_unit(const KParams& kp, const KtArgs& ka, con
 
 template <int D>
 __device__ __forceinline__ void kt_unit_any(const KParams& kp, const KtArgs& ka, int p, const double* As,
-                                            const int* tix, unsigned magic, unsigned char* dst) {
+                                            const int* tix, unsigned base, unsigned char* dst) {
   switch (p) {
-    case 0: kt_unit<D, 0>(kp, ka, As, tix, magic, dst); break;
-    case 1: kt_unit<D, 1>(kp, ka, As, tix, magic, dst); break;
-    case 2: if constexpr (npatterns(D) > 2) kt_unit<D, 2>(kp, ka, As, tix, magic, dst); break;
-    case 3: if constexpr (npatterns(D) > 3) kt_unit<D, 3>(kp, ka, As, tix, magic, dst); break;
-    case 4: if constexpr (npatterns(D) > 4) kt_unit<D, 4>(kp, ka, As, tix, magic, dst); break;
-    case 5: if constexpr (npatterns(D) > 4) kt_unit<D, 5>(kp, ka, As, tix, magic, dst); break;
-    case 6: if constexpr (npatterns(D) > 4) kt_unit<D, 6>(kp, ka, As, tix, magic, dst); break;
-    case 7: if constexpr (npatterns(D) > 4) kt_unit<D, 7>(kp, ka, As, tix, magic, dst); break;
+    case 0: kt_unit<D, 0>(kp, ka, As, tix, base, dst); break;
+    case 1: kt_unit<D, 1>(kp, ka, As, tix, base, dst); break;
+    case 2: if constexpr (npatterns(D) > 2) kt_unit<D, 2>(kp, ka, As, tix, base, dst); break;
+    case 3: if constexpr (npatterns(D) > 3) kt_unit<D, 3>(kp, ka, As, tix, base, dst); break;
+    case 4: if constexpr (npatterns(D) > 4) kt_unit<D, 4>(kp, ka, As, tix, base, dst); break;
+    case 5: if constexpr (npatterns(D) > 4) kt_unit<D, 5>(kp, ka, As, tix, base, dst); break;
+    case 6: if constexpr (npatterns(D) > 4) kt_unit<D, 6>(kp, ka, As, tix, base, dst); break;
+    case 7: if constexpr (npatterns(D) > 4) kt_unit<D, 7>(kp, ka, As, tix, base, dst); break;
     default:  // no tuples left: digits of zero
       const unsigned z[8] = {0x80808080u, 0x80808080u, 0x80808080u, 0x80808080u, 0x80808080u, 0x80808080u, 0x80808080u, 0x80808080u};
       for (int g = 0; g < 3; g++) kt_store8(dst + g * KT_AKG, KT_AD, z, z);
@@ -387,14 +391,14 @@ __global__ void __launch_bounds__(256) kt_prep_kernel(const __grid_constant__ KP
     E = KT_ELO;
   }
   if (q == 0) ka.wexp[((int64_t)yt * ka.nchunk + ch) * KT_COLS + y] = E | bad;
-  // largest |W| below 2^51, then shifted up by 3
-  const unsigned magic = (E + (2u << 20)) | 0x80000u;
+  // largest |W| below 2^53, then shifted up by 1
+  const unsigned base = E | 0xFFFFFu;
   for (int kg = q; kg < KT_CHUNK / 8; kg += 8) {
     unsigned z0[8], z1[8];
 #pragma unroll
     for (int e = 0; e < 8; e++) {
       int l0, l1;
-      kt_limbs(load(kg * 8 + e), magic, 3, l0, l1);
+      kt_limbs(load(kg * 8 + e), base, 1, l0, l1);
       kt_digits(l0, l1, z0[e], z1[e]);
     }
     unsigned char* dst = ka.wdig + (((int64_t)yt * ka.nchunk + ch) * 4 + kg / 6) * KT_WST + kg % 6 * KT_WKG + y * 16;
@@ -488,17 +492,26 @@ __global__ void __launch_bounds__(KT_THREADS, 1) kt_kernel(const __grid_constant
       const int* tix = sh.tix[c % 3];
       const double* As = row_of(tile);
       unsigned mx = 0;
+      // high words only (half the registers: 24 loads in flight)
+      const unsigned* hw = reinterpret_cast<const unsigned*>(As) + 1;
 #pragma unroll 1
-      for (int j = 0; j < 3; j++) {
-        constexpr int N = KT_CHUNK / 12;
-        double v[N];
-        kt_load<N>(As, kp.S, tix + quarter * (KT_CHUNK / 4) + j * N, v);
+      for (int j = 0; j < 2; j++) {
+        constexpr int N = KT_CHUNK / 8;
+        const int* te = tix + quarter * (KT_CHUNK / 4) + j * N;
+        unsigned v[N];
+#pragma unroll
+        for (int e = 0; e < N; e += 4) {
+          const int4 t = *reinterpret_cast<const int4*>(te + e);
+          v[e] = hw[2 * (int64_t)t.x * kp.S];
+          v[e + 1] = hw[2 * (int64_t)t.y * kp.S];
+          v[e + 2] = hw[2 * (int64_t)t.z * kp.S];
+          v[e + 3] = hw[2 * (int64_t)t.w * kp.S];
+        }
         unsigned m = 0;
 #pragma unroll
-        for (int e = 0; e < N; e++) m = max(m, (unsigned)__double2hiint(v[e]) & 0x7FFFFFFFu);
+        for (int e = 0; e < N; e++) m = max(m, v[e] & 0x7FFFFFFFu);
         if (m == 0) {  // zeros, or magnitudes below 2^-1042: the latter are out of range
-#pragma unroll
-          for (int e = 0; e < N; e++) m |= (unsigned)__double2loint(v[e]) != 0;
+          for (int e = 0; e < N; e++) m |= hw[2 * (int64_t)te[e] * kp.S - 1] != 0;
         }
         mx = max(mx, m);
       }
@@ -527,7 +540,7 @@ __global__ void __launch_bounds__(KT_THREADS, 1) kt_kernel(const __grid_constant
         if (tid < 32 && sh.colexp[c & 15][tid] >> 31) sh.bad[it & 7] = 1;
         if (quarter == 0) sh.rowexp[c & 7][row] = E;
         // largest |A| below 2^(bits - up)
-        const unsigned magic = (E + ((unsigned)(53 - ka.bits + ka.up) << 20)) | 0x80000u;
+        const unsigned base = (E + ((unsigned)(53 - ka.bits + ka.up) << 20)) | 0xFFFFFu;
         const int ns = stages_of(ch);
         for (int j = 0; ok && j < ns; j++, n++) {
           if ((n & 1) != group) continue;  // the other group's stage
@@ -539,7 +552,7 @@ __global__ void __launch_bounds__(KT_THREADS, 1) kt_kernel(const __grid_constant
             bulk_g2s(st + KT_ND * KT_AD, wd + ((int64_t)ch * 4 + j) * KT_WST, KT_WST, &sh.st_full[n & 1]);
           }
           const int u = 2 * j + half;
-          kt_unit_any<D>(kp, ka, sh.pat[c % 3][u], As, tix + u * KT_UNIT, magic, st + half * 3 * KT_AKG + row * 16);
+          kt_unit_any<D>(kp, ka, sh.pat[c % 3][u], As, tix + u * KT_UNIT, base, st + half * 3 * KT_AKG + row * 16);
           kt_proxy_fence();
           mbar_arrive(&sh.st_full[n & 1]);
         }
@@ -699,7 +712,7 @@ inline cudaMemPool_t kt_pool(int dev) {
 
 // Whether KT takes the contraction: exact arithmetic with integer coefficients
 // (the operator's 1-norm is then at most 127, so the limb sums stay below 2^31),
-// and at least four row tiles. Smaller calls stay with KC, whose FP64 sums equal
+// and more than two row tiles. Smaller calls stay with KC, whose FP64 sums equal
 // those of the summation followed by the contraction alone bit for bit.
 template <int D>
 bool launch_kt(const KParams& kp, const double* W, int64_t Y, int64_t ldw, double* C, int64_t ldc, cudaStream_t st,
@@ -712,7 +725,7 @@ bool launch_kt(const KParams& kp, const double* W, int64_t Y, int64_t ldw, doubl
   }
   int64_t T = 1;
   for (int k = 0; k < D; k++) T *= kp.O;
-  if (T < 1 || T > 0x7FFFFFFF || kp.S < 4 * KT_ROWS || (kp.flags & KF_ALPHA_MUL) || L > 127) return false;
+  if (T < 1 || T > 0x7FFFFFFF || kp.S <= 2 * KT_ROWS || (kp.flags & KF_ALPHA_MUL) || L > 127) return false;
   int lg = 0;
   while ((double)(1 << lg) < L) lg++;
   KtArgs ka{};
@@ -724,7 +737,7 @@ bool launch_kt(const KParams& kp, const double* W, int64_t Y, int64_t ldw, doubl
   ka.ytiles = (int)((Y + KT_COLS - 1) / KT_COLS);
   ka.tiles = (kp.S + KT_ROWS - 1) / KT_ROWS * ka.ytiles;
   ka.bits = 54 - lg;
-  ka.up = ka.bits > 51 ? ka.bits - 51 : 0;  // the rounding addition holds 51 bits
+  ka.up = ka.bits > 53 ? ka.bits - 53 : 0;  // a mantissa has 53 bits
   // kp.cexp = (53 - 2 W + kdrop + aexp) << 20 + 0x80000, aexp = the coefficients' scale;
   // a joined sum counts 2^56 of the products' units 2^(E_A + 1 - bits + aexp) 2^(E_W - 53)
   const int aexp = ((kp.cexp - 0x80000) >> 20) - 53 + 2 * kp.W - kp.kdrop;

@@ -33,10 +33,10 @@ def _tol(A, d, coef, W):
     return (1e-14 + 2 * T * 2.0 ** -53) * chain_norm(d, coef, True) * np.abs(A).max() * np.abs(W).sum(axis=1).max()
 
 
-# d, spectators (S = 512, 513, 516, several tiles per CTA), O (a partial unit, a
+# d, spectators (S = 257, 512, 513, 516, several tiles per CTA), O (a partial unit, a
 # partial stage, an exact chunk, several chunks), columns
 CASES = [
-    (3, (8, 8, 8), 4, 1, 1), (3, (513, 1, 1), 5, 2, 31), (3, (8, 16, 4), 6, 1, 32), (3, (43, 12, 1), 13, "random", 33),
+    (3, (257, 1, 1), 6, 1, 5), (3, (8, 8, 8), 4, 1, 1), (3, (513, 1, 1), 5, 2, 31), (3, (8, 16, 4), 6, 1, 32), (3, (43, 12, 1), 13, "random", 33),
     (3, (33, 32, 31), 3, 3, 65), (2, (32, 16), 12, "pair", 5), (2, (129, 5), 30, "pair", 40),
     (4, (2, 3, 4, 25), 3, 5, 7), (4, (8, 8, 8, 1), 5, "random", 32), (4, (129, 1, 5, 1), 6, 6, 3),
 ]
