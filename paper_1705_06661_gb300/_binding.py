@@ -72,9 +72,11 @@ def _load() -> ctypes.CDLL:
     lib = ctypes.CDLL(path)
     sig = [ctypes.c_int, _I64P, _VP, _I64P, _VP, _I64P, _VP, ctypes.c_int, ctypes.c_int, ctypes.c_double,
            ctypes.c_double, ctypes.c_int, _VP]
+    # (the address arrays of these as plain addresses: see _call)
+    ssig = [_VP if t is _I64P else t for t in sig]
     for name in ("spinsum_2d", "spinsum_3d", "spinsum_4d"):
         f = getattr(lib, name)
-        f.argtypes = sig
+        f.argtypes = ssig
         f.restype = ctypes.c_int
     hsig = sig[:-1] + [_VP, ctypes.c_size_t, _VP]
     for name in ("spinsum_2d_host", "spinsum_3d_host", "spinsum_4d_host"):
@@ -124,21 +126,35 @@ def _check(status: int) -> int:
     return status
 
 
+_ARRAYS = [ctypes.c_int64 * n for n in range(9)]
+
+
 def _i64(a) -> ctypes.Array:
     a = [int(x) for x in a]
-    return (ctypes.c_int64 * len(a))(*a)
+    return (_ARRAYS[len(a)] if len(a) < 9 else ctypes.c_int64 * len(a))(*a)
 
 
 def _coef(coef) -> np.ndarray:
+    if type(coef) is np.ndarray and coef.dtype == np.float64 and coef.flags.c_contiguous:
+        return coef
     return np.ascontiguousarray(np.asarray(coef, dtype=np.float64))
+
+
+_SHAPES = {n: ctypes.c_int64 * (3 * n) for n in (4, 6, 8)}
 
 
 def _call(fn, n, dtype, ext, A, lda, B, ldb, coef, nfactors, mode, alpha, beta, inplace, stream):
     if len(ext) != n or len(lda) != n or len(ldb) != n:
         raise ValueError(f"expected {n} extents and strides")
     c = _coef(coef)
-    return _check(fn(int(dtype), _i64(ext), _VP(A), _i64(lda), _VP(B), _i64(ldb), _VP(c.ctypes.data),
-                     int(nfactors), int(mode), float(alpha), float(beta), int(inplace), _VP(stream)))
+    # extents and strides in one array: a small call's time is mostly this marshalling
+    try:
+        s = _SHAPES[n](*ext, *lda, *ldb)
+    except TypeError:
+        s = _SHAPES[n](*[int(x) for x in (*ext, *lda, *ldb)])
+    p = ctypes.addressof(s)
+    return _check(fn(int(dtype), p, A, p + 8 * n, B, p + 16 * n, c.__array_interface__["data"][0], int(nfactors),
+                     int(mode), float(alpha), float(beta), int(inplace), stream))
 
 
 def spinsum_unpack(d, dtype, ext, P, ldp, B, ldb, stream) -> int:

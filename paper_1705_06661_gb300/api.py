@@ -19,8 +19,11 @@ from . import _binding as _b
 def colmajor_empty(shape, dtype=torch.float64, device="cuda") -> torch.Tensor:
     """Dense column-major tensor (first index fastest) with logical shape `shape`."""
     shape = tuple(int(s) for s in shape)
-    t = torch.empty(tuple(reversed(shape)), dtype=dtype, device=device)
-    return t.permute(*reversed(range(len(shape))))
+    strides, n = [], 1
+    for s in shape:
+        strides.append(n)
+        n *= max(s, 1)
+    return torch.empty_strided(shape, strides, dtype=dtype, device=device)
 
 
 def colmajor_like(x: torch.Tensor) -> torch.Tensor:
@@ -34,6 +37,9 @@ def to_colmajor(x: torch.Tensor) -> torch.Tensor:
 
 
 def _coef_chain(coef, d: int) -> np.ndarray:
+    if type(coef) is np.ndarray and coef.ndim == 2 and coef.dtype == np.float64 and coef.flags.c_contiguous \
+            and coef.shape[1] == _FACT[d]:
+        return coef
     c = np.asarray(coef.detach().cpu().numpy() if isinstance(coef, torch.Tensor) else coef, dtype=np.float64)
     if c.ndim == 1:
         c = c[None, :]
@@ -42,14 +48,30 @@ def _coef_chain(coef, d: int) -> np.ndarray:
     return np.ascontiguousarray(c)
 
 
+_FACT = [math.factorial(k) for k in range(5)]
+
+
+# the current stream's handle without building a Stream object, where torch offers it
+_current_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None) or (
+    lambda index: torch.cuda.current_stream(index).cuda_stream)
+
+
+def _raw_stream(stream, device: torch.device) -> int:
+    """The CUDA stream handle to launch on: `stream`, or the device's current one."""
+    return _current_raw_stream(device.index) if stream is None else stream.cuda_stream
+
+
 def _dims(x: torch.Tensor, d: int):
     """extents and element strides in ABI order (d spectators, d permuted);
     a tensor with only the d permuted dimensions gets spectator extents 1."""
     if x.dim() == 2 * d:
-        return list(x.shape), list(x.stride())
+        return x.shape, x.stride()
     if x.dim() == d:
         return [1] * d + list(x.shape), [1] * d + list(x.stride())
     raise ValueError(f"expected a tensor with {d} or {2 * d} dimensions, got {x.dim()}")
+
+
+_SUMS = {2: _b.spinsum_2d, 3: _b.spinsum_3d, 4: _b.spinsum_4d}
 
 
 def spinsum(A: torch.Tensor, coef, *, d: int | None = None, out: torch.Tensor | None = None,
@@ -62,11 +84,12 @@ def spinsum(A: torch.Tensor, coef, *, d: int | None = None, out: torch.Tensor | 
         d = A.dim() // 2
     if d not in (2, 3, 4):
         raise ValueError("d must be 2, 3 or 4")
-    if not A.is_cuda:
+    device, torch_dtype = A.device, A.dtype
+    if device.type != "cuda":
         raise ValueError("A must be a CUDA tensor")
-    if A.dtype == torch.float64:
+    if torch_dtype is torch.float64:
         dtype = _b.SPINSUM_F64
-    elif A.dtype == torch.float32:
+    elif torch_dtype is torch.float32:
         dtype = _b.SPINSUM_F32
     else:
         raise TypeError("A must be float64 or float32")
@@ -77,16 +100,19 @@ def spinsum(A: torch.Tensor, coef, *, d: int | None = None, out: torch.Tensor | 
         out = colmajor_like(A) if beta == 0.0 else None
         if out is None:
             raise ValueError("beta != 0 needs an output tensor")
-    if out.dtype != A.dtype or out.device != A.device or tuple(out.shape) != tuple(A.shape):
+    elif out.dtype is not torch_dtype or out.device != device or out.shape != A.shape:
         raise ValueError("out must match A in dtype, device and shape")
     ext, lda = _dims(A, d)
-    _, ldb = _dims(out, d)
+    ldb = lda if out is A else _dims(out, d)[1]
     mode = (_b.SPINSUM_FACTORIZED if factorized else _b.SPINSUM_EXPANDED) | (_b.SPINSUM_ADJOINT if adjoint else 0) \
         | (_b.SPINSUM_STRICT if strict else 0) | (_b.SPINSUM_TMA if tma else 0)
-    st = (stream or torch.cuda.current_stream(A.device)).cuda_stream
-    fn = {2: _b.spinsum_2d, 3: _b.spinsum_3d, 4: _b.spinsum_4d}[d]
-    with torch.cuda.device(A.device):
-        fn(dtype, ext, A.data_ptr(), lda, out.data_ptr(), ldb, c, c.shape[0], mode, alpha, beta, int(inplace), st)
+    args = (dtype, ext, A.data_ptr(), lda, out.data_ptr(), ldb, c, c.shape[0], mode, alpha, beta, inplace,
+            _raw_stream(stream, device))
+    if torch.cuda.current_device() == device.index:
+        _SUMS[d](*args)
+    else:
+        with torch.cuda.device(device):
+            _SUMS[d](*args)
     return out
 
 
