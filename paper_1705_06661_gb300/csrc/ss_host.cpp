@@ -511,7 +511,13 @@ int plan_one(const Request& r, Launch* L) {
       // (d = 4 through the Klein four-group transform: SS_K1_POS4, measured best
       // with the L2 prefetch of the next chunk)
       const int64_t pos = (d == 4 && (kp.flags & KF_WHT)) ? SS_K1_POS4 : 8192;
-      const int64_t cpb0 = std::min<int64_t>(kp.nchunk, std::max<int64_t>(1, pos / per));
+      int64_t cpb0 = std::min<int64_t>(kp.nchunk, std::max<int64_t>(1, pos / per));
+      // few orbits: enough blocks for about four rounds of the resident CTAs (O = 6 has 56
+      // orbits for d = 3; 336 blocks of 8192 positions left half the SMs idle)
+      int64_t orbits = 0;
+      for (int p = 0; p < np; p++) orbits += kp.norb[p];
+      const int64_t min_bpo = (SS_K1_MINBLOCKS + orbits - 1) / std::max<int64_t>(orbits, 1);
+      cpb0 = std::min(cpb0, std::max<int64_t>(1, kp.nchunk / min_bpo));
       const int64_t nbo = (kp.nchunk + cpb0 - 1) / cpb0;
       kp.cpb = (int)((kp.nchunk + nbo - 1) / nbo);
       const int64_t bpo = (kp.nchunk + kp.cpb - 1) / kp.cpb;
@@ -1010,7 +1016,7 @@ struct spinsum_plan {
   unsigned char* d_image = nullptr;  // device copy of the batch image (owned)
   ImageShape shape{};
   int cpb_scale = 3;                 // chunks per block = 2^cpb_scale
-  int order = 0;                     // 0 as given, 1 largest problems first
+  int order = 0;                     // 0 as given, 1 largest problems first, 2 a launch per problem
   int occ = 1;                       // grid = SMs * max blocks per SM / occ
   std::string desc;
 };
@@ -1050,12 +1056,38 @@ int plan_build(spinsum_plan* P, int cpb_scale, int order, int occ, cudaStream_t 
   return SPINSUM_OK;
 }
 
+// Whether a plan may run as a chain of single-problem launches: every batched
+// problem is one of the d <= 3 kernels that can overlap their ends.
+bool plan_chainable(const spinsum_plan* P) {
+  for (const Launch& L : P->launches)
+    if (L.kernel != 1 && L.kernel != 3 && (L.kernel != 0 || L.kp.nspec > 3)) return false;
+  return true;
+}
+
 int plan_launch(spinsum_plan* P, cudaStream_t st) {
+  if (P->order == 2) {
+    // A launch per problem, each allowed to start under the end of the one before it.
+    // The batched kernel reads its parameters from shared memory and takes every block
+    // from a counter; K1 has them as constants. 32 uneven 3D blocks of 24 MB to 1.6 GB, FP64:
+    // 3563 us batched, 3054 us chained; of 15 to 70 MB, the batched kernel stays ahead (147 us),
+    // so the tuner times both.
+    int flags = KF_CHAIN;
+    for (const Launch& L0 : P->launches) {
+      if (L0.kernel != 0) continue;
+      Launch L = L0;
+      L.kp.status = status_ptr();
+      L.kp.flags |= flags;
+      flags = KF_CHAIN | KF_CHAIN_NEXT;
+      const cudaError_t e = launch_k1(L.kp.nspec, L.kp, L.ar, L.vec, st);
+      t_launches++;
+      if (e != cudaSuccess) return cuda_fail(e, "chained kernel launch");
+    }
+  }
   const KParams* probs = reinterpret_cast<const KParams*>(P->d_image + P->shape.probs);
   const int64_t* prefix = reinterpret_cast<const int64_t*>(P->d_image + P->shape.prefix);
   const int* vec = reinterpret_cast<const int*>(P->d_image + P->shape.vec);
   unsigned long long* ctr = reinterpret_cast<unsigned long long*>(P->d_image + P->shape.ctr);
-  for (size_t k = 0; k < P->classes.size(); k++) {
+  for (size_t k = 0; k < P->classes.size() && P->order != 2; k++) {
     const ClassRange& c = P->classes[k];
     cudaError_t e = launch_kb(c.d, c.ar, probs + c.first, prefix + c.pfirst, vec + c.first, c.n, ctr + 2 * k,
                               P->grid[k], st, nullptr);
@@ -1162,6 +1194,7 @@ int spinsum_plan_create(spinsum_plan** plan, const spinsum_problem* problems, in
   for (auto& kv : tune_cache())
     if (kv.first == key) {
       best[0] = kv.second[0]; best[1] = kv.second[1]; best[2] = kv.second[2];
+      if (best[1] == 2 && !plan_chainable(P)) best[1] = 0;  // (the key does not tell every layout)
       cached = true;
     }
   const bool any_k1 = P->general.size() < P->launches.size();
@@ -1170,9 +1203,11 @@ int spinsum_plan_create(spinsum_plan** plan, const spinsum_problem* problems, in
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
     float best_ms = 1e30f;
+    const int orders = plan_chainable(P) ? 3 : 2;
     for (int cs = 0; cs <= 5; cs++)
-      for (int order = 0; order <= 1; order++)
+      for (int order = 0; order < orders; order++)
         for (int occ = 1; occ <= 2; occ++) {
+          if (order == 2 && (cs != 3 || occ != 1)) continue;  // these do not matter to the chain
           int rc = plan_build(P, cs, order, occ, st);
           if (rc != SPINSUM_OK) { cudaEventDestroy(e0); cudaEventDestroy(e1); plan_free(P); delete P; return rc; }
           float ms = 1e30f;
@@ -1200,7 +1235,7 @@ int spinsum_plan_create(spinsum_plan** plan, const spinsum_problem* problems, in
   snprintf(buf, sizeof buf,
            "problems=%zu classes=%zu general=%zu blocks=%lld chunks_per_block=%d order=%s occupancy=1/%d%s",
            P->launches.size(), P->classes.size(), P->general.size(), (long long)blocks, 1 << best[0],
-           best[1] ? "largest-first" : "as-given", best[2],
+           best[1] == 2 ? "launch-per-problem" : (best[1] ? "largest-first" : "as-given"), best[2],
            cached ? " (cached)" : (allow_tuning_runs ? " (tuned)" : " (heuristic)"));
   P->desc = buf;
   *plan = P;

@@ -349,6 +349,10 @@ constexpr int MP_MAX = MP_TOTAL_4;
 #ifndef SS_K1_KB0F32
 #define SS_K1_KB0F32 2
 #endif
+// K1: blocks that a problem of few orbits is cut into
+#ifndef SS_K1_MINBLOCKS
+#define SS_K1_MINBLOCKS 2432
+#endif
 // K1, d = 4 transform path: spectator positions per member per block
 #ifndef SS_K1_POS4
 #define SS_K1_POS4 5120
@@ -383,6 +387,8 @@ enum {
   KF_BETA = 1,        // beta != 0: read B_old
   KF_ALPHA_MUL = 2,   // exact path: alpha is not a power of two, multiply at the end
   KF_KDROP = 4,       // exact path: round the fixed-point sum before conversion
+  KF_CHAIN = 16,      // K1, d <= 3: one of a plan's launches that may overlap (see launch_k1_bt)
+  KF_CHAIN_NEXT = 32, // ... and not the first of them
   KF_WHT = 8,         // exact path, d = 4: freely transformable orbits through the Klein four-group transform
 };
 

@@ -344,27 +344,6 @@ __device__ __forceinline__ void k2_fill(const KParams& kp, const int (&val)[4], 
   if (u == 0) dsc.allfull = part == 0;
 }
 
-// Colex unranking as in unrank(), by a whole warp at once: the candidates c of
-// each position are tested 32 at a time (C(c, i + 1) grows with c, so the
-// qualifying c form a prefix and the answer is its last element). Every lane
-// returns the same tuple; all 32 lanes must be active.
-template <int ND>
-__device__ __forceinline__ void unrank_warp(int64_t r, int O, int (&v)[4]) {
-  const int lane = threadIdx.x & 31;
-#pragma unroll
-  for (int i = ND - 1; i >= 0; i--) {
-    int cnt = 0;
-    for (int c0 = i; c0 < O; c0 += 32) {
-      const int c = c0 + lane;
-      const unsigned m = __ballot_sync(0xffffffffu, c < O && binom(c, i + 1) <= r);
-      cnt += __popc(m);
-      if (m != 0xffffffffu) break;
-    }
-    v[i] = i + cnt - 1;
-    r -= binom(v[i], i + 1);
-  }
-}
-
 // Work ids and block orbits. Block orbits are visited in groups: the sorted
 // tuple c of coarse blocks (F tiles per edge, F = 2^k2lf) is unranked from
 // id / F^d as a multiset (colex rank of the strictly increasing c_k + k), and

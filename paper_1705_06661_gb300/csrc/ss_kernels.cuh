@@ -73,6 +73,27 @@ __device__ __forceinline__ void unrank(int64_t r, int O, int* v) {
   }
 }
 
+// Colex unranking as in unrank(), by a whole warp at once: the candidates c of
+// each position are tested 32 at a time (C(c, i + 1) grows with c, so the
+// qualifying c form a prefix and the answer is its last element). Every lane
+// returns the same tuple; all 32 lanes must be active.
+template <int ND>
+__device__ __forceinline__ void unrank_warp(int64_t r, int O, int (&v)[4]) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int i = ND - 1; i >= 0; i--) {
+    int cnt = 0;
+    for (int c0 = i; c0 < O; c0 += 32) {
+      const int c = c0 + lane;
+      const unsigned m = __ballot_sync(0xffffffffu, c < O && binom(c, i + 1) <= r);
+      cnt += __popc(m);
+      if (m != 0xffffffffu) break;
+    }
+    v[i] = i + cnt - 1;
+    r -= binom(v[i], i + 1);
+  }
+}
+
 __device__ __forceinline__ unsigned long long shr64(unsigned long long x, unsigned k) {
   unsigned long long r;
   asm("shr.b64 %0, %1, %2;" : "=l"(r) : "l"(x), "r"(k));  // amounts >= 64 give 0
@@ -575,7 +596,9 @@ __device__ __forceinline__ void k1_body(const KParams& kp, int64_t orb, int64_t 
   __syncthreads();
   if (threadIdx.x < 32) {
     int val[4] = {0, 0, 0, 0};
-    unrank<Pat<D, P>::ND>(orb, kp.O, val);
+    // (the batched kernel and d = 4, at their register limits, search serially)
+    if constexpr (D <= 3 && BT != 2) unrank_warp<Pat<D, P>::ND>(orb, kp.O, val);
+    else unrank<Pat<D, P>::ND>(orb, kp.O, val);
 #pragma unroll
     for (int u = 0; u < M; u++) {
       if (threadIdx.x == (u & 31)) {
@@ -820,16 +843,40 @@ __device__ __forceinline__ void k1_block(const KParams& kp, int64_t b) {
 template <int D, int AR, int VEC, typename T, int XW = 0, int BT = 2>
 __global__ void __launch_bounds__(256, (D == 4 && AR == AR_EXACT) ? (XW ? SS_4DW_MINBLOCKS : SS_4D_MINBLOCKS) : 1)
     k1_kernel(const __grid_constant__ KParams kp) {
+  if constexpr (D <= 3) {
+    // the next launch of the chain may start as soon as this one's CTAs all have
+    if (kp.flags & KF_CHAIN) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  }
   k1_block<D, AR, VEC, T, XW, D <= 3 ? SS_K1_KBMAX3 : SS_K1_KBMAX4, k1_kb0<D, AR, VEC>(), BT>(kp, blockIdx.x);
+  if constexpr (D <= 3) {
+    // this launch is complete only after the one before it: what follows the last
+    // launch in the stream then follows all of them
+    if (kp.flags & KF_CHAIN_NEXT) asm volatile("griddepcontrol.wait;" ::: "memory");
+  }
 }
 
-// single problems: with and without the beta term as two kernels (in one,
-// the old values' registers cost the beta = 0 path a resident CTA)
+// Single problems: with and without the beta term as two kernels (in one, the old
+// values' registers cost the beta = 0 path a resident CTA). A launch with
+// KF_CHAIN_NEXT may start under the end of the one before it in the stream
+// (programmatic dependent launch), whose problem it shares no data with.
 template <int D, int AR, int VEC, typename T>
 void launch_k1_bt(const KParams& kp, cudaStream_t st) {
   const dim3 grid((unsigned)kp.pre[npatterns(D)]), block(256);
-  if (kp.flags & KF_BETA) k1_kernel<D, AR, VEC, T, 0, 1><<<grid, block, 0, st>>>(kp);
-  else k1_kernel<D, AR, VEC, T, 0, 0><<<grid, block, 0, st>>>(kp);
+  auto fn = kp.flags & KF_BETA ? k1_kernel<D, AR, VEC, T, 0, 1> : k1_kernel<D, AR, VEC, T, 0, 0>;
+  if (kp.flags & KF_CHAIN_NEXT) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.stream = st;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, fn, kp);
+  } else {
+    fn<<<grid, block, 0, st>>>(kp);
+  }
 }
 
 // ---------------------------------------------------------------------------
