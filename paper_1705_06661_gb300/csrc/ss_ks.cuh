@@ -11,8 +11,8 @@
 // unit-stride stores: each element crosses HBM once each way. The general
 // kernel KG reads and writes the same elements as scattered 8-byte accesses,
 // unranks a tuple per thread and sums with FP64 instructions: 2480 us on
-// A[32^3, 12^3], factorized Table II row 1 (0.37 TB/s), against 470 us here (507 with one
-// buffer per CTA).
+// A[32^3, 12^3], factorized Table II row 1 (0.37 TB/s), against 396 us here (507 with one
+// buffer per CTA, 470 with the multiplication by alpha predicated into the common path).
 //
 // - Canonical tuples come from a table in shared memory, grouped by equality
 //   pattern and built once per CTA, so warps run one pattern's code and no
@@ -30,7 +30,10 @@
 
 namespace ss {
 
-constexpr int AR_FIXED = 4;  // kernel-template choice of this file: FP64 through fixed_sum
+// kernel-template choices of this file: FP64 through fixed_sum, and the same with an alpha that is
+// no power of two (one kernel for both would issue the multiplication, predicated off, on the
+// FP64 pipe, the busiest one)
+constexpr int AR_FIXED = 4, AR_FIXED_MUL = 5;
 
 struct KsArgs {
   int ns;             // spectator positions per round
@@ -213,11 +216,9 @@ __device__ __forceinline__ void ks_group(const KParams& kp, const KsArgs& ka, un
     T x[M];
 #pragma unroll
     for (int u = 0; u < M; u++) x[u] = sm[ks_slot<D, P>(ka, u, val)];
-    if constexpr (AR == AR_FIXED) {
-      // (alpha not a power of two occurs for d <= 3 only: see ks_plan)
-      const bool mul = D <= 3 && (kp.flags & KF_ALPHA_MUL);
+    if constexpr (AR == AR_FIXED || AR == AR_FIXED_MUL) {
       auto sink = [&](int u, double y) {
-        if (D <= 3 && mul) y = __dmul_rn(kp.alpha, y);
+        if constexpr (AR == AR_FIXED_MUL) y = __dmul_rn(kp.alpha, y);
         sm[ks_slot<D, P>(ka, u, val)] = y;
       };
       if (!fixed_sum<D, P>(kp, ka, x, sink)) ks_strict_group<D, P>(kp, ka, tup, sm);
@@ -381,6 +382,8 @@ __global__ void __launch_bounds__(NT, MINB) ks_kernel(const __grid_constant__ KP
 constexpr int KS_SMEM_MAX = 227 * 1024 - 1024;
 // shared memory a round's blocks aim at: three CTAs per SM with two buffers each;
 // larger blocks take one position per round, and one buffer where two do not fit
+// (A[32^3,12^3] FP64: 396 us; CTAs of 128 threads, six or eight per SM, 400 and 413; four CTAs of
+// 256 threads at 64 registers 455)
 constexpr int KS_SMEM_AIM = 32 * 1024;
 
 // Whether the problem has KS's layout (permuted strides 1, O, .., O^(d-1) in
@@ -502,8 +505,9 @@ bool launch_ks(const KParams& kp, int ar, cudaStream_t st, cudaError_t* e) {
     else *e = launch_ks_impl<4, AR_FIXED, 256, 2, double>(kp, ka, smem, st);
   } else {
     if (ar == AR_F32) *e = launch_ks_impl<D, AR_F32, 256, 5, float>(kp, ka, smem, st);
-    else if (ar == AR_EXACT && fixed) *e = launch_ks_impl<D, AR_FIXED, 256, 3, double>(kp, ka, smem, st);
-    else *e = launch_ks_impl<D, AR_STRICT, 256, 3, double>(kp, ka, smem, st);
+    else if (ar != AR_EXACT || !fixed) *e = launch_ks_impl<D, AR_STRICT, 256, 3, double>(kp, ka, smem, st);
+    else if (kp.flags & KF_ALPHA_MUL) *e = launch_ks_impl<D, AR_FIXED_MUL, 256, 3, double>(kp, ka, smem, st);
+    else *e = launch_ks_impl<D, AR_FIXED, 256, 3, double>(kp, ka, smem, st);
   }
   return true;
 }
