@@ -512,7 +512,7 @@ int plan_one(const Request& r, Launch* L) {
       // with the L2 prefetch of the next chunk)
       const int64_t pos = (d == 4 && (kp.flags & KF_WHT)) ? SS_K1_POS4 : 8192;
       int64_t cpb0 = std::min<int64_t>(kp.nchunk, std::max<int64_t>(1, pos / per));
-      // few orbits: enough blocks for about four rounds of the resident CTAs (O = 6 has 56
+      // few orbits: enough blocks for about three rounds of the resident CTAs (O = 6 has 56
       // orbits for d = 3; 336 blocks of 8192 positions left half the SMs idle)
       int64_t orbits = 0;
       for (int p = 0; p < np; p++) orbits += kp.norb[p];
@@ -1069,7 +1069,7 @@ int plan_launch(spinsum_plan* P, cudaStream_t st) {
     // A launch per problem, each allowed to start under the end of the one before it.
     // The batched kernel reads its parameters from shared memory and takes every block
     // from a counter; K1 has them as constants. 32 uneven 3D blocks of 24 MB to 1.6 GB, FP64:
-    // 3563 us batched, 3054 us chained; of 15 to 70 MB, the batched kernel stays ahead (147 us),
+    // 3563 us batched, 2990 us chained; of 15 to 70 MB, the batched kernel stays ahead (147 us),
     // so the tuner times both.
     int flags = KF_CHAIN;
     for (const Launch& L0 : P->launches) {

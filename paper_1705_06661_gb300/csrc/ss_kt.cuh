@@ -69,7 +69,7 @@ struct KtArgs {
   int ytiles;
   int nchunk;
   int upre[9];         // unit prefix per pattern
-  int bits, up;        // |A| < 2^bits: rounded to 2^(bits - up) and shifted up
+  int bits;            // |A| < 2^bits on its grid
   int sh0;             // exponent of a joined sum's unit, less the two scales' exponents
   int opow[4];
   // prepared by kt_prep_kernel in the call's workspace
@@ -131,18 +131,19 @@ __device__ __forceinline__ bool kt_sync(bool ok) {
 }
 
 // x on the grid of a scale as two limbs l1 2^24 + l0 of a signed integer, shifted up by
-// `up`: the mantissa shifted right by (base - |x|'s high word) >> 20 places (base: the
+// UP: the mantissa shifted right by (base - |x|'s high word) >> 20 places (base: the
 // scale's exponent field, plus the places that the grid drops, with 20 ones below it).
 // (One FP64 addition of 1.5 * 2^52 grid units does the same in five instructions, but at
 // two FP64 operations per SM and clock: 2509 against 2275 us on A[48^3,16^3].)
-__device__ __forceinline__ void kt_limbs(double x, unsigned base, int up, int& l0, int& l1) {
+template <int UP>
+__device__ __forceinline__ void kt_limbs(double x, unsigned base, int& l0, int& l1) {
   const unsigned xh = (unsigned)__double2hiint(x), xl = (unsigned)__double2loint(x);
   const unsigned k = (base - (xh & 0x7FFFFFFFu)) >> 20;
   const unsigned long long mant = ((unsigned long long)((xh & 0x000FFFFFu) | 0x00100000u) << 32) | xl;
   const long long q = (long long)shr64(mant, k);
   const long long X = (int)xh < 0 ? -q : q;
-  l0 = (int)(((unsigned)X << up) & 0xFFFFFFu);
-  l1 = (int)(X >> (24 - up));
+  l0 = (int)(((unsigned)X << UP) & 0xFFFFFFu);
+  l1 = (int)(X >> (24 - UP));
 }
 
 // limbs y1 2^24 + y0 -> the biased digits: byte 3..0 of z1, then byte 2..0 of z0, each digit + 128
@@ -200,7 +201,7 @@ __device__ __forceinline__ void kt_unit(const KParams& kp, const KtArgs& ka, con
     int l0[M], l1[M];
 #pragma unroll
     for (int v = 0; v < M; v++) {
-      kt_limbs(x[v], base, ka.up, l0[v], l1[v]);
+      kt_limbs<0>(x[v], base, l0[v], l1[v]);
     }
 #pragma unroll
     for (int g = 0; g < 3; g++) {
@@ -235,7 +236,7 @@ __device__ __forceinline__ void kt_unit(const KParams& kp, const KtArgs& ka, con
     int l0[M], l1[M], y0[M], y1[M];
 #pragma unroll
     for (int v = 0; v < M; v++) {
-      kt_limbs(x[o * M % NB + v], base, ka.up, l0[v], l1[v]);
+      kt_limbs<0>(x[o * M % NB + v], base, l0[v], l1[v]);
     }
     if constexpr (P == 0) {
 #pragma unroll
@@ -398,7 +399,7 @@ __global__ void __launch_bounds__(256) kt_prep_kernel(const __grid_constant__ KP
 #pragma unroll
     for (int e = 0; e < 8; e++) {
       int l0, l1;
-      kt_limbs(load(kg * 8 + e), base, 1, l0, l1);
+      kt_limbs<1>(load(kg * 8 + e), base, l0, l1);
       kt_digits(l0, l1, z0[e], z1[e]);
     }
     unsigned char* dst = ka.wdig + (((int64_t)yt * ka.nchunk + ch) * 4 + kg / 6) * KT_WST + kg % 6 * KT_WKG + y * 16;
@@ -539,8 +540,8 @@ __global__ void __launch_bounds__(KT_THREADS, 1) kt_kernel(const __grid_constant
         }
         if (tid < 32 && sh.colexp[c & 15][tid] >> 31) sh.bad[it & 7] = 1;
         if (quarter == 0) sh.rowexp[c & 7][row] = E;
-        // largest |A| below 2^(bits - up)
-        const unsigned base = (E + ((unsigned)(53 - ka.bits + ka.up) << 20)) | 0xFFFFFu;
+        // largest |A| below 2^bits
+        const unsigned base = (E + ((unsigned)(53 - ka.bits) << 20)) | 0xFFFFFu;
         const int ns = stages_of(ch);
         for (int j = 0; ok && j < ns; j++, n++) {
           if ((n & 1) != group) continue;  // the other group's stage
@@ -736,8 +737,7 @@ bool launch_kt(const KParams& kp, const double* W, int64_t Y, int64_t ldw, doubl
   ka.ldc = ldc;
   ka.ytiles = (int)((Y + KT_COLS - 1) / KT_COLS);
   ka.tiles = (kp.S + KT_ROWS - 1) / KT_ROWS * ka.ytiles;
-  ka.bits = 54 - lg;
-  ka.up = ka.bits > 53 ? ka.bits - 53 : 0;  // a mantissa has 53 bits
+  ka.bits = lg > 0 ? 54 - lg : 53;  // a mantissa has 53 bits
   // kp.cexp = (53 - 2 W + kdrop + aexp) << 20 + 0x80000, aexp = the coefficients' scale;
   // a joined sum counts 2^56 of the products' units 2^(E_A + 1 - bits + aexp) 2^(E_W - 53)
   const int aexp = ((kp.cexp - 0x80000) >> 20) - 53 + 2 * kp.W - kp.kdrop;
