@@ -21,10 +21,9 @@
 //   chosen so that all d! permuted reads fall on 16 different bank pairs
 //   (tests/test_k2t_cpu.py checks every permutation).
 //
-// FP64, factorized Table II rows 1 and 5: A[544]^3 590 -> 416 us (6.2 TB/s, 0.91 of the
-// copy; bound by DRAM and, next, FP64 and issue), A[112]^4 1084 -> 707 us (3.6 TB/s; the
-// unrolled sums of 24 members miss the instruction cache, and 48 KB block orbits leave room
-// for four in flight per SM).
+// FP64, factorized Table II rows 1 and 5: A[544]^3 590 -> 412 us (6.2 TB/s, 0.92 of the
+// copy; bound by DRAM and, next, FP64 and issue), A[112]^4 1084 -> 563 us (4.5 TB/s; 48 KB
+// block orbits leave room for four in flight per SM: the sums wait for loads).
 //
 // TMA needs 16-byte strides (even extents for FP64); other tensors, the beta
 // term, strict order, dense d = 4 operators and d = 2 (two 8 KB tiles per block
@@ -93,54 +92,25 @@ constexpr K2TTab<D> make_k2ttab() {
 template <int D>
 __device__ constexpr K2TTab<D> kK2TTab = make_k2ttab<D>();
 
-// element pattern EP: for member u the first permutation that gives it
-template <int D, int EP>
-struct K2TMember {
-  int n[24] = {};
-  int tau[24][4] = {};
-};
-template <int D, int EP>
-constexpr K2TMember<D, EP> make_k2tmember() {
-  K2TMember<D, EP> r{};
-  const Pattern<D> pe = make_pattern<D>(EP);
-  const Sym<D> S = make_sym<D>();
-  for (int u = 0; u < pe.m; u++) {
-    int t = -1;
-    for (int n = 0; n < fact(D) && t < 0; n++) {
-      bool same = true;
-      for (int k = 0; k < D; k++) same = same && pe.lab[0][S.p[n][k]] == pe.lab[u][k];
-      if (same) t = n;
-    }
-    r.n[u] = t;
-    for (int k = 0; k < D; k++) r.tau[u][k] = S.p[t][k];
-  }
-  return r;
-}
-template <int D, int EP>
-__device__ constexpr K2TMember<D, EP> kK2TMember = make_k2tmember<D, EP>();
+// member u of an element orbit: permutation u (lexicographic)
+template <int D>
+__device__ constexpr Sym<D> kK2TSym = make_sym<D>();
 
-// the canonical offsets of a degenerate block orbit grouped by element pattern,
-// as K2List but in K2TShape's order
+// the canonical offsets of a degenerate block orbit (some block coordinates equal:
+// sorted within them), packed one byte per index
 template <int D, int BP>
 constexpr K2List<D> make_k2tlist() {
   using K = K2TShape<D>;
   K2List<D> r{};
   const Pattern<D> pb = make_pattern<D>(BP);
-  for (int ep = 0; ep < npatterns(D); ep++)
-    for (int e0 = 0; e0 < K::NT; e0++) {
-      int w[4] = {0, 0, 0, 0};
-      K::elem(e0, w);
-      bool ok = true;
-      unsigned eq = 0;
-      for (int k = 0; k + 1 < D; k++)
-        if (pb.lab[0][k] == pb.lab[0][k + 1]) {
-          ok = ok && w[k] <= w[k + 1];
-          if (w[k] == w[k + 1]) eq |= 1u << k;
-        }
-      if (!ok || k2_elem_pattern<D>(eq) != ep) continue;
-      r.e[r.n++] = (unsigned)w[0] | ((unsigned)w[1] << 8) | ((unsigned)w[2] << 16) | ((unsigned)w[3] << 24 & 0x1F000000u) |
-                   ((unsigned)ep << 29);
-    }
+  for (int e0 = 0; e0 < K::NT; e0++) {
+    int w[4] = {0, 0, 0, 0};
+    K::elem(e0, w);
+    bool ok = true;
+    for (int k = 0; k + 1 < D; k++)
+      if (pb.lab[0][k] == pb.lab[0][k + 1]) ok = ok && w[k] <= w[k + 1];
+    if (ok) r.e[r.n++] = (unsigned)w[0] | (unsigned)w[1] << 8 | (unsigned)w[2] << 16 | (unsigned)w[3] << 24;
+  }
   return r;
 }
 template <int D, int BP>
@@ -165,81 +135,76 @@ struct K2TShared {
   unsigned bin[D][K2T_BIN];         // C(c, k + 1)
 };
 
-// in-tile place of offset w o tau
-template <int D, int EP>
+// in-tile place of offset w o (permutation u)
+template <int D>
 __device__ __forceinline__ int k2t_lin(int u, const int (&w)[4]) {
   constexpr int SH = D == 3 ? 3 : 2;
   int a = 0;
 #pragma unroll
-  for (int k = 0; k < D; k++) a += w[kK2TMember<D, EP>.tau[u][k]] << (SH * k);
+  for (int k = 0; k < D; k++) a += w[kK2TSym<D>.p[u][k]] << (SH * k);
   return a;
 }
 
 // the strict core for a group outside the fixed-point range, out of line
-template <int D, int EP>
+template <int D>
 static __device__ __noinline__ void k2t_strict_group(const KParams& kp, unsigned pk, const int* tb, double* sm) {
-  constexpr int M = Pat<D, EP>::M;
-  const int w[4] = {(int)(pk & 255), (int)(pk >> 8 & 255), (int)(pk >> 16 & 255), (int)(pk >> 24 & 31)};
+  constexpr int M = fact(D);
+  const int w[4] = {(int)(pk & 255), (int)(pk >> 8 & 255), (int)(pk >> 16 & 255), (int)(pk >> 24)};
   double x[M];
 #pragma unroll
-  for (int u = 0; u < M; u++) x[u] = sm[tb[kK2TMember<D, EP>.n[u]] + k2t_lin<D, EP>(u, w)];
-  strict_core<D, EP>(kp, x);
+  for (int u = 0; u < M; u++) x[u] = sm[tb[u] + k2t_lin<D>(u, w)];
+  strict_core<D, 0>(kp, x);
 #pragma unroll
-  for (int u = 0; u < M; u++) sm[tb[kK2TMember<D, EP>.n[u]] + k2t_lin<D, EP>(u, w)] = __dmul_rn(kp.alpha, x[u]);
+  for (int u = 0; u < M; u++) sm[tb[u] + k2t_lin<D>(u, w)] = __dmul_rn(kp.alpha, x[u]);
 }
 
-// one element orbit. GEN: of a generic block orbit, whose tile n is permutation n's
-template <int D, int EP, int AR, bool GEN, typename T>
+// One element orbit, always through the operator on all d! permutations: where
+// indices are equal, members coincide, each is read and written by this thread as
+// often as permutations give it, and every copy gets the same value (the sums over the
+// permutations are the pattern's own, term by term). A body per equality pattern, as
+// in K2, made 75 KB of code for d = 4: "no instruction" was the second largest stall
+// (A[112]^4 687 us; one body for all 24-member orbits 584; one for everything 563).
+// GEN: of a generic block orbit, whose tile n is permutation n's.
+template <int D, int AR, bool GEN, typename T>
 __device__ __forceinline__ void k2t_group(const KParams& kp, unsigned pk, const int (&w)[4], const int* tb, T* sm) {
-  constexpr int M = Pat<D, EP>::M;
-  auto slot = [&](int u) {
-    return (GEN ? kK2TMember<D, EP>.n[u] * K2TShape<D>::NT : tb[kK2TMember<D, EP>.n[u]]) + k2t_lin<D, EP>(u, w);
-  };
+  constexpr int M = fact(D);
+  auto slot = [&](int u) { return (GEN ? u * K2TShape<D>::NT : tb[u]) + k2t_lin<D>(u, w); };
   T x[M];
 #pragma unroll
   for (int u = 0; u < M; u++) x[u] = sm[slot(u)];
   if constexpr (AR == AR_F32) {
     T y[M];
-    apply_group<D, EP, AR_F32, T>(kp, x, y);
+    apply_group<D, 0, AR_F32, T>(kp, x, y);
 #pragma unroll
     for (int u = 0; u < M; u++) sm[slot(u)] = y[u];
-  } else if constexpr (D == 4 && wht_ok<EP>()) {
+  } else if constexpr (D == 4) {
     auto sink = [&](int u, double v, int) { sm[slot(u)] = v; };
-    if (!exact_core_wht4<EP>(kp, x, sink)) k2t_strict_group<D, EP>(kp, pk, tb, sm);
+    if (!exact_core_wht4<0>(kp, x, sink)) k2t_strict_group<D>(kp, pk, tb, sm);
   } else {
     T y[M];
-    if (exact_core<D, EP>(kp, x, y)) {
-      const bool mul = D == 3 && (kp.flags & KF_ALPHA_MUL);
-      if (mul) {
+    if (exact_core<D, 0>(kp, x, y)) {
+      if (kp.flags & KF_ALPHA_MUL) {
 #pragma unroll
         for (int u = 0; u < M; u++) y[u] = __dmul_rn(kp.alpha, y[u]);
       }
 #pragma unroll
       for (int u = 0; u < M; u++) sm[slot(u)] = y[u];
     } else {
-      k2t_strict_group<D, EP>(kp, pk, tb, sm);
+      k2t_strict_group<D>(kp, pk, tb, sm);
     }
   }
 }
 
+// the element orbits at offsets list[0..n), or (no list) at the thread's own offset pk0
 template <int D, int AR, typename T>
-__device__ __forceinline__ void k2t_degenerate(const KParams& kp, const K2TStage& st, const unsigned* list, int n, T* sm) {
+__device__ __forceinline__ void k2t_listed(const KParams& kp, const K2TStage& st, const unsigned* list, int n, unsigned pk0,
+                                           T* sm) {
 #pragma unroll 1
   for (int i = threadIdx.x; i < n; i += 256) {
-    const unsigned pk = list[i];
-    const int w[4] = {(int)(pk & 255), (int)(pk >> 8 & 255), (int)(pk >> 16 & 255), (int)(pk >> 24 & 31)};
-    const int wl = D == 3 ? w[2] : w[3];
-    if (wl >= st.lim) continue;
-    switch (pk >> 29) {
-      case 0: k2t_group<D, 0, AR, false, T>(kp, pk, w, st.tb, sm); break;
-      case 1: k2t_group<D, 1, AR, false, T>(kp, pk, w, st.tb, sm); break;
-      case 2: k2t_group<D, 2, AR, false, T>(kp, pk, w, st.tb, sm); break;
-      case 3: k2t_group<D, 3, AR, false, T>(kp, pk, w, st.tb, sm); break;
-      case 4: if constexpr (npatterns(D) > 4) k2t_group<D, 4, AR, false, T>(kp, pk, w, st.tb, sm); break;
-      case 5: if constexpr (npatterns(D) > 4) k2t_group<D, 5, AR, false, T>(kp, pk, w, st.tb, sm); break;
-      case 6: if constexpr (npatterns(D) > 4) k2t_group<D, 6, AR, false, T>(kp, pk, w, st.tb, sm); break;
-      case 7: if constexpr (npatterns(D) > 4) k2t_group<D, 7, AR, false, T>(kp, pk, w, st.tb, sm); break;
-    }
+    const unsigned pk = list ? list[i] : pk0;
+    const int w[4] = {(int)(pk & 255), (int)(pk >> 8 & 255), (int)(pk >> 16 & 255), (int)(pk >> 24)};
+    if (w[D - 1] >= st.lim) continue;
+    k2t_group<D, AR, false, T>(kp, pk, w, st.tb, sm);
   }
 }
 
@@ -348,18 +313,19 @@ __global__ void __launch_bounds__(K2T_THREADS, MINB)
       const K2TStage& st = sh.st[s];
       const int bp = st.bp;
       T* const sm = buf + s * SE;
-      if (bp == 0) {
+      if (D == 3 && bp == 0) {
+        // the generic block orbit's tile offsets as constants: a second copy of the six
+        // members' code, which is small
 #pragma unroll 1
         for (int e = 0; e < K::NT; e += 256) {
-          int w[4] = {w0[0], w0[1], w0[2], w0[3]};
-          if constexpr (D == 3) w[2] ^= (e >> 8) << 2;  // bit 8 of the element index
-          const int wl = D == 3 ? w[2] : w[3];
-          if (wl < st.lim)
-            k2t_group<D, 0, AR, true, T>(kp, (unsigned)(w[0] | w[1] << 8 | w[2] << 16 | w[3] << 24), w, st.tb, sm);
+          const int w[4] = {w0[0], w0[1], w0[2] ^ (e >> 8) << 2, 0};  // bit 8 of the element index
+          if (w[2] < st.lim)
+            k2t_group<D, AR, D == 3, T>(kp, (unsigned)(w[0] | w[1] << 8 | w[2] << 16), w, st.tb, sm);
         }
-      } else if (bp > 0) {
-        const unsigned* list = kK2TList<D, 1>.e;
-        int n = kK2TList<D, 1>.n;
+      } else if (bp >= 0) {
+        const unsigned* list = nullptr;
+        int n = K::NT;
+        if (bp == 1) { list = kK2TList<D, 1>.e; n = kK2TList<D, 1>.n; }
         if (bp == 2) { list = kK2TList<D, 2>.e; n = kK2TList<D, 2>.n; }
         if (bp == 3) { list = kK2TList<D, 3>.e; n = kK2TList<D, 3>.n; }
         if constexpr (D == 4) {
@@ -368,7 +334,7 @@ __global__ void __launch_bounds__(K2T_THREADS, MINB)
           if (bp == 6) { list = kK2TList<D, 6>.e; n = kK2TList<D, 6>.n; }
           if (bp == 7) { list = kK2TList<D, 7>.e; n = kK2TList<D, 7>.n; }
         }
-        k2t_degenerate<D, AR, T>(kp, st, list, n, sm);
+        k2t_listed<D, AR, T>(kp, st, list, n, (unsigned)(w0[0] | w0[1] << 8 | w0[2] << 16 | w0[3] << 24), sm);
       }
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // before the TMA store reads the stage
       __syncwarp();
