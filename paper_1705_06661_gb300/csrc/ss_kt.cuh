@@ -713,8 +713,13 @@ inline cudaMemPool_t kt_pool(int dev) {
 
 // Whether KT takes the contraction: exact arithmetic with integer coefficients
 // (the operator's 1-norm is then at most 127, so the limb sums stay below 2^31),
-// and more than two row tiles. Smaller calls stay with KC, whose FP64 sums equal
-// those of the summation followed by the contraction alone bit for bit.
+// more than two row tiles (smaller calls stay with KC, whose FP64 sums equal those of
+// the summation followed by the contraction alone bit for bit), and where it is the
+// faster one. Per spectator position KT costs 4.9 ps per tuple of its whole chunks and 32
+// columns, KC 1.8 ps per tuple and column of its column tiles (A[48^3,16^3]: KT 2.23 ms up to
+// 32 columns, KC 3.4 ms up to 4; A[100,90,80,6^3], 216 tuples in two chunks: KT 1.34 ms, KC
+// 1.08 ms up to 4 columns and 2.09 up to 8); and below a million tuple-columns both are shorter
+// than the call, KC with one launch and no workspace.
 template <int D>
 bool launch_kt(const KParams& kp, const double* W, int64_t Y, int64_t ldw, double* C, int64_t ldc, cudaStream_t st,
                cudaError_t* e) {
@@ -753,6 +758,8 @@ bool launch_kt(const KParams& kp, const double* W, int64_t Y, int64_t ldw, doubl
   if (units > 100000000) return false;
   for (int p = npatterns(D); p < 9; p++) ka.upre[p] = (int)units;
   ka.nchunk = (int)((units + KT_UPC - 1) / KT_UPC);
+  const int64_t ct = Y <= 4 ? 4 : (Y <= 8 ? 8 : (Y <= 16 || D == 4 ? 16 : 32)), kc_cols = (Y + ct - 1) / ct * ct;
+  if (2.7 * KT_CHUNK * ka.nchunk * ka.ytiles > (double)T * kc_cols || (double)kp.S * T * kc_cols < 1e6) return false;
   ka.opow[0] = 1;
   for (int k = 1; k < 4; k++) ka.opow[k] = k < D ? ka.opow[k - 1] * kp.O : 0;
   static DeviceCache cache;  // SMs, after raising the kernel's shared-memory limit
@@ -779,7 +786,7 @@ bool launch_kt(const KParams& kp, const double* W, int64_t Y, int64_t ldw, doubl
                 bp = (int64_t)ka.nchunk * KT_UPC * 4;
   unsigned char* ws = nullptr;
   cudaMemPool_t pool = kt_pool(dev);
-  if (!pool || ka.ytiles > 65535 || cudaMallocFromPoolAsync((void**)&ws, (size_t)(bw + be + bt + bp), pool, st) != cudaSuccess) {
+  if (!pool || ka.ytiles > 65535 || bw > (2LL << 30) || cudaMallocFromPoolAsync((void**)&ws, (size_t)(bw + be + bt + bp), pool, st) != cudaSuccess) {
     cudaGetLastError();
     return false;  // KC needs no workspace
   }
