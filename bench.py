@@ -159,9 +159,10 @@ def measured_peaks():
 # DRAM-traffic figure is used only while these are unchanged)
 KERNEL_SOURCES = {
     "k1": ("ss_internal.h", "ss_kernels.cuh", "ss_k1_d3.cu", "ss_k1_d4_exact.cu", "ss_host.cpp", "ss_status.cu"),
-    "k2": ("ss_internal.h", "ss_kernels.cuh", "ss_k2.cuh", "ss_k2_d3.cu", "ss_k2_d4_exact.cu", "ss_host.cpp",
-           "ss_status.cu"),
-    "kc": ("ss_internal.h", "ss_kernels.cuh", "ss_contract.cuh", "ss_kc_d3.cu", "ss_host.cpp", "ss_status.cu"),
+    "k2": ("ss_internal.h", "ss_kernels.cuh", "ss_tma.cuh", "ss_k2.cuh", "ss_k2t.cuh", "ss_k2_d3.cu", "ss_k2t_d3.cu",
+           "ss_k2_d4_exact.cu", "ss_k2t_d4.cu", "ss_host.cpp", "ss_status.cu"),
+    "kc": ("ss_internal.h", "ss_kernels.cuh", "ss_tma.cuh", "ss_contract.cuh", "ss_kt.cuh", "ss_kc_d3.cu",
+           "ss_host.cpp", "ss_status.cu"),
 }
 CASE_KERNEL = {"3d": "k1", "3d-small": "k1", "4d": "k1", "4d-small": "k1", "paper-3d": "k2", "paper-4d": "k2",
                "paper-3d-544": "k2", "paper-4d-112": "k2",
@@ -360,8 +361,9 @@ def extra_cases_contract(ss, wl, dev, stream, A, B, coef):
     C[s, y] = sum_t S(A)[s, t] W[y, t] on the benchmark tensor (S(A) never
     stored), against the unfused pair (the summation into B, then the
     contraction kernel alone on B) and, for context, cuBLAS DGEMM for the
-    contraction alone. Both kernels are bound by the FP64 pipe (Y multiply-adds
-    per element of A); the fused call saves the write and re-read of S(A)."""
+    contraction alone. The fused call runs on the tensor cores (exact digit
+    products); the contraction alone is bound by the FP64 pipe (Y multiply-adds
+    per element of A)."""
     import torch
     out = []
     spec = tuple(A.shape[:3])
@@ -375,6 +377,7 @@ def extra_cases_contract(ss, wl, dev, stream, A, B, coef):
         C = ss.colmajor_empty(spec + (Y,), device=dev)
         reps = 5 if Y <= 32 else 2
         torch.matmul(W.permute(1, 0).t(), Braw)      # cuBLAS's first call on this shape sets up; not timed
+        ss.contract(A, coef, W, out=C, factorized=True)   # the first call maps the workspace pool; not timed
         fused, _ = best_of(lambda: ss.contract(A, coef, W, out=C, factorized=True), reps, stream)
         summ, _ = best_of(lambda: ss.spinsum(A, coef, d=3, out=B, factorized=True), reps, stream)
         plain, _ = best_of(lambda: ss.contract(B, None, W, out=C), reps, stream)
@@ -386,8 +389,7 @@ def extra_cases_contract(ss, wl, dev, stream, A, B, coef):
                     "unfused_parts_ms": [round(summ * 1e3, 3), round(plain * 1e3, 3)],
                     "speedup_vs_unfused": round((summ + plain) / fused, 3),
                     "cublas_dgemm_contraction_only_ms": round(cublas * 1e3, 3),
-                    "fp64_TFLOPs": round(tf, 3), "bound": "fp64",
-                    "frac_of_nominal_fp64": round(tf / 1.25, 3)})
+                    "fp64_equivalent_TFLOPs": round(tf, 3), "bound": "instruction issue"})
         del W, C
     return out
 
