@@ -183,12 +183,22 @@ int spinsum_4d_host(int dtype, const int64_t ext[8], const void* A, const int64_
  *          never read; must not overlap A or W.
  * stream : cudaStream_t to launch on.
  *
- * Every element of S(A) is formed in registers (the cores of spinsum_3d, so
- * with the exact core S(A) equals what spinsum_3d/4d would store) and
- * multiplied into FP64 accumulators in orbit order; A is read once per group
- * of 16 columns of C. FP64 only. Errors: SPINSUM_ERR_ARG (bad d, extents,
+ * S(A) is formed on chip and never stored. FP64 only. With integer
+ * coefficients (up to a common power of two, sum |a| <= 127), without STRICT,
+ * from 257 spectator positions on and where it is faster, the products run on
+ * the tensor cores: S(A) and W as 55-bit integers on one power-of-two scale per
+ * row resp. column and chunk of 192 tuples, every product and sum exact in
+ * integers, one rounding to FP64 per chunk; tiles with infinities, NaN or
+ * magnitudes beyond 2^+-440 are summed in FP64. Otherwise S(A) equals what
+ * spinsum_3d/4d would store and is multiplied into FP64 accumulators in orbit
+ * order. Either way |dC| <= (1e-14 + 2 O^d 2^-53) sum|a| max|A| max_y sum_t |W|.
+ * The tensor-core path takes a stream-ordered workspace (W's digits, 448
+ * bytes per tuple and 32 columns) from a pool of the library that keeps at
+ * most 32 MB between calls; where none can be had the FP64 path runs. Under
+ * stream capture the workspace becomes allocation and free nodes of the graph.
+ * Errors: SPINSUM_ERR_ARG (bad d, extents,
  * leading dimensions, pointers or mode bits), SPINSUM_ERR_ALIAS (C overlaps A
- * or W), SPINSUM_ERR_CUDA. Asynchronous on `stream`; allocates nothing.
+ * or W), SPINSUM_ERR_CUDA. Asynchronous on `stream`.
  */
 int spinsum_contract(int d, const int64_t ext[], const void* A, const double* coef, int nfactors, int mode,
                      const void* W, int64_t Y, int64_t ldw, void* C, int64_t ldc, spinsum_stream_t stream);
@@ -226,7 +236,8 @@ int spinsum_pack(int d, int dtype, const int64_t ext[], const void* B, const int
 
 /*
  * Batched plans: many independent spin summations (uneven extents, mixed d,
- * mixed coefficient sets) run by one persistent kernel launch. The plan's work
+ * mixed coefficient sets) run by one persistent kernel launch or a chain of
+ * overlapping ones. The plan's work
  * list is the GPU form of the task-based scheduling of Sec. 4.5 (Algorithm
  * 5a): every (problem, block of orbits) pair is a task, and the persistent
  * CTAs take tasks in a fixed order instead of from a dynamic queue.
@@ -240,7 +251,9 @@ int spinsum_pack(int d, int dtype, const int64_t ext[], const void* B, const int
  * candidates on `stream` and may therefore run the problems: inputs must be
  * valid and in-place problems are restored only if `allow_tuning_runs` is 0,
  * in which case a fixed heuristic is used). dtype applies to all problems.
- * spinsum_plan_execute launches the whole batch as one kernel on `stream`;
+ * spinsum_plan_execute launches the whole batch as one kernel per (d,
+ * arithmetic) class on `stream`, or, where the autotuner measured it faster,
+ * as a launch per problem that may overlap with the end of the one before it;
  * it allocates nothing and may be captured in a CUDA graph. The kernel's CTAs
  * take work from counters in the plan's device memory (the last CTA of a
  * launch resets them), so two executions of one plan must not overlap on the

@@ -1,5 +1,6 @@
 #pragma once
-// KC: the spin summation fused into the contraction it feeds (Sec. 1: the
+// KC: the spin summation fused into the contraction it feeds, in FP64 (ss_kt.cuh has
+// the tensor-core form, for integer coefficients and larger calls) (Sec. 1: the
 // spin-summed intermediates of CC theory enter tensor contractions; Sec. 6).
 //
 //   C[s, y] = sum_t S(A)[s, t] * W[y, t]   (SUM = true)
