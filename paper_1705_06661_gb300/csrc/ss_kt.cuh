@@ -539,17 +539,26 @@ __global__ void __launch_bounds__(KT_THREADS, 1) kt_kernel(const __grid_constant
         const int* tix = sh.tix[c % 3];
         const unsigned short* rm = &sh.rowmax[c & 3][0][row];
         unsigned E = max(max(rm[0], rm[KT_ROWS]), max(rm[2 * KT_ROWS], rm[3 * KT_ROWS])) << 20;
+        bool bad = false;
         if (E < KT_ELO || E > KT_EHI) {
-          if (E != 0) sh.bad[it & 7] = 1;
+          bad = E != 0;
           E = KT_ELO;
         }
-        if (tid < 32 && sh.colexp[c & 15][tid] >> 31) sh.bad[it & 7] = 1;
-        if (quarter == 0) sh.rowexp[c & 7][row] = E;
+        if (half == 0) bad |= row < KT_COLS && sh.colexp[c & 15][row] >> 31;
         // largest |A| below 2^bits
         const unsigned base = (E + ((unsigned)(53 - ka.bits) << 20)) | 0xFFFFFu;
         const int ns = stages_of(ch);
         for (int j = 0; ok && j < ns; j++, n++) {
           if ((n & 1) != group) continue;  // the other group's stage
+          // The epilogue reads the scales and the flag behind acc_full, which follows the
+          // arrivals of the groups that filled the chunk's stages, and of no other: a chunk of
+          // one stage orders one group's writes only. So the group that fills a stage
+          // publishes them, ahead of its arrival. (A stage's buffer was free two stages ago, so
+          // the epilogue is at most five chunks behind, within the rings of eight.)
+          if (half == 0) {
+            sh.rowexp[c & 7][row] = E;
+            if (bad) sh.bad[it & 7] = 1;
+          }
           unsigned char* st = kt_smem + (n & 1) * KT_STAGE;
           const int u = 2 * j + half;
           double x0[12];
