@@ -88,7 +88,7 @@ struct KtShared {
   alignas(16) int tix[3][KT_CHUNK];  // tuple indices of a chunk (no tuple left: 0, and W's digits are 0)
   int pat[3][KT_UPC];            // pattern of each unit, -1: none
   int bad[8];                    // by tile mod 8: a scale is out of range
-  uint64_t tab_full[3], tab_empty[3], mx_full[2], st_full[2], st_empty[2], acc_full[2], acc_empty[2], drain;
+  uint64_t tab_full[3], tab_empty[3], mx_full[2], st_full[2], w_full[2], st_empty[2], acc_full[2], acc_empty[2], drain;
   uint32_t tmem;
 };
 
@@ -459,7 +459,8 @@ __global__ void __launch_bounds__(KT_THREADS, 1) kt_kernel(const __grid_constant
     }
     for (int i = 0; i < 2; i++) {
       mbar_init(&sh.mx_full[i], KT_PROD);
-      mbar_init(&sh.st_full[i], KT_PROD / 2 + 1);  // a group, and W's copy
+      mbar_init(&sh.st_full[i], KT_PROD / 2);  // a group
+      mbar_init(&sh.w_full[i], 1);             // W's copy
       mbar_init(&sh.st_empty[i], 1);
       mbar_init(&sh.acc_full[i], 1);
       mbar_init(&sh.acc_empty[i], 128);
@@ -527,6 +528,7 @@ __global__ void __launch_bounds__(KT_THREADS, 1) kt_kernel(const __grid_constant
       return true;
     };
     int c = 0, n = 0, it = 0;  // chunks, stages and tiles so far
+    int copies = 0;            // of W, by this thread
     if (blockIdx.x < ka.tiles) ok = maxima(blockIdx.x, 0);
     for (int64_t tile = blockIdx.x; ok && tile < ka.tiles; tile += step, it++) {
       const double* As = row_of(tile);
@@ -566,8 +568,9 @@ __global__ void __launch_bounds__(KT_THREADS, 1) kt_kernel(const __grid_constant
           ok = mbar_wait(&sh.st_empty[n & 1], ((n >> 1) & 1) ^ 1, lim);
           if (!ok) break;
           if ((tid & 255) == 0) {
-            mbar_arrive_expect_tx(&sh.st_full[n & 1], KT_WST);
-            bulk_g2s(st + KT_ND * KT_AD, wd + ((int64_t)ch * 4 + j) * KT_WST, KT_WST, &sh.st_full[n & 1]);
+            mbar_arrive_expect_tx(&sh.w_full[group], KT_WST);
+            bulk_g2s(st + KT_ND * KT_AD, wd + ((int64_t)ch * 4 + j) * KT_WST, KT_WST, &sh.w_full[group]);
+            copies++;
           }
           kt_unit_any<D>(kp, ka, sh.pat[c % 3][u], As, tix + u * KT_UNIT, base, st + half * 3 * KT_AKG + row * 16, x0);
           kt_proxy_fence();
@@ -576,6 +579,9 @@ __global__ void __launch_bounds__(KT_THREADS, 1) kt_kernel(const __grid_constant
         mbar_arrive(&sh.tab_empty[c % 3]);
       }
     }
+    // no copy is in flight when the CTA's shared memory is given up, also where a wait ran
+    // out (the copy before the last has landed: its stage was used and freed)
+    if (copies > 0) ok = mbar_wait(&sh.w_full[group], (copies - 1) & 1, kDrainLimit) && ok;
   } else if (warp < MMA_WARP) {
     // ---- epilogue: join the digit sums of a chunk, add up the chunks ----
     const int row = tid - KT_PROD;
@@ -652,7 +658,10 @@ __global__ void __launch_bounds__(KT_THREADS, 1) kt_kernel(const __grid_constant
           const uint32_t acc = tmem + (uint32_t)(c & 1) * 256;
           const int ns = stages_of(ch);
           for (int j = 0; j < ns; j++, n++) {
-            if (!mbar_wait(&sh.st_full[n & 1], (n >> 1) & 1, lim)) { ok = false; break; }
+            if (!mbar_wait(&sh.st_full[n & 1], (n >> 1) & 1, lim) || !mbar_wait(&sh.w_full[n & 1], (n >> 1) & 1, lim)) {
+              ok = false;
+              break;
+            }
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             const uint32_t sa = sbase + (n & 1) * KT_STAGE, sw = sa + KT_ND * KT_AD;
             for (int ks = 0; ks < 3; ks++)
@@ -667,9 +676,10 @@ __global__ void __launch_bounds__(KT_THREADS, 1) kt_kernel(const __grid_constant
           }
           if (ok) kt_commit(&sh.acc_full[c & 1]);
         }
-      // no matrix instruction is in flight when the accumulators are given back
+      // no matrix instruction is in flight when the accumulators are given back, also where
+      // a wait ran out
       kt_commit(&sh.drain);
-      ok = mbar_wait(&sh.drain, 0, lim) && ok;
+      ok = mbar_wait(&sh.drain, 0, kDrainLimit) && ok;
     }
     __syncwarp();
   } else if (warp == MMA_WARP + 1) {
