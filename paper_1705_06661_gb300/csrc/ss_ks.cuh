@@ -389,8 +389,8 @@ constexpr int KS_SMEM_AIM = 32 * 1024;
 // Whether the problem has KS's layout (permuted strides 1, O, .., O^(d-1) in
 // some order, the same in A and B) and its block fits on chip; fills ka and
 // the CTA's shared-memory bytes. Below O^d = 64 the rows are too short to be
-// worth staging, and FP64 with d = 4 needs the transform's weights (KF_WHT) for
-// AR_FIXED, else the FP64 order runs.
+// worth staging. *fixed: the problem has an AR_FIXED form (FP64 with d = 4 needs the
+// transform's weights, KF_WHT, for it).
 inline bool ks_plan(int d, const KParams& kp, int es, KsArgs* ka, int* smem, bool* fixed) {
   const int64_t O = kp.O;
   int64_t T = 1;
@@ -464,6 +464,30 @@ inline bool ks_plan(int d, const KParams& kp, int es, KsArgs* ka, int* smem, boo
   return true;
 }
 
+// Whether KS is faster than KG, which takes a thread per orbit and position: a CTA of KS
+// builds its tables (O^d places, the tuples) and takes whole blocks, so a call of few
+// positions leaves SMs idle behind CTAs that mostly prepare. Measured over S = 1 .. 98304,
+// inputs not in L2 where larger (KS / KG, us):
+//   d = 2, fixed or FP32: O = 16, S = 1024 8.6 / 6.8, 2048 9.3 / 11.0; O = 64, S = 256 30 / 24,
+//     512 38 / 42; O = 128, S = 1 140 / 8.5, 256 164 / 124, 512 205 / 242; FP32 alike;
+//     strict (FP64 pipe in both): O = 32, S = 4096 67 / 64, 16384 237 / 324.
+//   d = 3, fixed: O = 8, S = 64 10.8 / 10.1, 512 11.1 / 16.2; O = 20, S = 64 26 / 24, 128
+//     27 / 38; O = 27, S = 64 64 / 42, 128 66 / 78. FP32: O = 8, S = 1024 9.2 / 8.8, 2048
+//     10.0 / 13.6; O = 24, S = 256 39 / 39, 512 54 / 75. Strict: O = 12, S = 4096 400 / 235.
+//   d = 4, fixed: O = 3, S = 16 16 / 48, 4096 16 / 43; O = 12, S = 1 42 / 68, 1024 270 / 1240.
+//     FP32 (KG holds its own while the tensors stay in L2): O = 8, S = 2048 170 / 131, 8192
+//     638 / 829; O = 12, S = 256 71 / 70, 1024 223 / 409. Strict: O = 8, S = 1024 573 / 262.
+inline bool ks_faster(int d, bool f32, bool fixed, int64_t S, int64_t O, int64_t T) {
+  const int64_t N = S * T;
+  if (d == 2) {
+    if (!f32 && !fixed) return N >= 9000000;
+    return N >= 520000 && S >= (O < 80 ? 520 : 340);
+  }
+  if (f32) return d == 3 ? N >= 650000 && S >= 250 : N >= 11000000;
+  if (!fixed) return false;
+  return d == 4 || T < 3000 || S >= 96;
+}
+
 template <int D, int AR, int NT, int MINB, typename T>
 cudaError_t launch_ks_impl(const KParams& kp, const KsArgs& ka, int smem, cudaStream_t st) {
   auto fn = ks_kernel<D, AR, NT, MINB, T>;
@@ -496,18 +520,19 @@ bool launch_ks(const KParams& kp, int ar, cudaStream_t st, cudaError_t* e) {
   int smem = 0;
   bool fixed = false;
   if (!ks_plan(D, kp, ar == AR_F32 ? 4 : 8, &ka, &smem, &fixed)) return false;
+  fixed = fixed && ar == AR_EXACT;
+  if (!ks_faster(D, ar == AR_F32, fixed, kp.S, kp.O, ka.T)) return false;
   if constexpr (D == 4) {
     // 24-member groups take 128 registers: two CTAs of 256 threads, or, where a
     // block leaves room for one CTA only, one of 512
     if (ar == AR_F32) *e = launch_ks_impl<4, AR_F32, 256, 2, float>(kp, ka, smem, st);
-    else if (!(ar == AR_EXACT && fixed)) *e = launch_ks_impl<4, AR_STRICT, 256, 2, double>(kp, ka, smem, st);
     else if (smem > KS_SMEM_MAX / 2) *e = launch_ks_impl<4, AR_FIXED, 512, 1, double>(kp, ka, smem, st);
     else *e = launch_ks_impl<4, AR_FIXED, 256, 2, double>(kp, ka, smem, st);
   } else {
     if (ar == AR_F32) *e = launch_ks_impl<D, AR_F32, 256, 5, float>(kp, ka, smem, st);
-    else if (ar != AR_EXACT || !fixed) *e = launch_ks_impl<D, AR_STRICT, 256, 3, double>(kp, ka, smem, st);
-    else if (kp.flags & KF_ALPHA_MUL) *e = launch_ks_impl<D, AR_FIXED_MUL, 256, 3, double>(kp, ka, smem, st);
-    else *e = launch_ks_impl<D, AR_FIXED, 256, 3, double>(kp, ka, smem, st);
+    else if (fixed && (kp.flags & KF_ALPHA_MUL)) *e = launch_ks_impl<D, AR_FIXED_MUL, 256, 3, double>(kp, ka, smem, st);
+    else if (fixed) *e = launch_ks_impl<D, AR_FIXED, 256, 3, double>(kp, ka, smem, st);
+    else if constexpr (D == 2) *e = launch_ks_impl<D, AR_STRICT, 256, 3, double>(kp, ka, smem, st);
   }
   return true;
 }
