@@ -23,17 +23,24 @@
 // - KG's FP64 arithmetic is native FP64 in the reference order; GB300's FP64
 //   pipe (2 operations per SM per clock) limits that to 57 G elements/s on the
 //   three-factor-term chains. Here the sums run in 64-bit integers on a grid
-//   fine enough that the result is more accurate than the FP64 sum (fixed_sum
-//   below); groups outside its range, and SPINSUM_STRICT, take the FP64 order.
+//   fine enough that the result is as accurate as the FP64 sum (fixed_sum
+//   below); groups outside its range, groups of an operator with zero
+//   coefficients whose magnitudes are too far apart, and SPINSUM_STRICT take
+//   the FP64 order.
+#include <algorithm>
+#include <array>
+#include <cmath>
+
 #include "ss_devcache.h"
 #include "ss_k2.cuh"
 
 namespace ss {
 
-// kernel-template choices of this file: FP64 through fixed_sum, and the same with an alpha that is
+// kernel-template choices of this file: FP64 through fixed_sum; the same with an alpha that is
 // no power of two (one kernel for both would issue the multiplication, predicated off, on the
-// FP64 pipe, the busiest one)
-constexpr int AR_FIXED = 4, AR_FIXED_MUL = 5;
+// FP64 pipe, the busiest one); and with fixed_sum's guard, for operators with zero coefficients,
+// any alpha (compiled into the first, unused: A[32^3,12^3] 404 us against 396)
+constexpr int AR_FIXED = 4, AR_FIXED_MUL = 5, AR_FIXED_GUARD = 6;
 
 struct KsArgs {
   int ns;             // spectator positions per round
@@ -49,6 +56,9 @@ struct KsArgs {
   int bits;           // AR_FIXED: an input's magnitude stays below 2^bits
   int sh0;            // AR_FIXED: result exponent offset (see fixed_sum)
   unsigned emin, emax;
+  int supp[8];        // AR_FIXED: fewest inputs of an output of pattern p; 0: all of them
+  int guard;          // AR_FIXED: some of supp are not 0
+  unsigned below;     // AR_FIXED: an input this far (exponent field) below the largest is small
 };
 
 // quotient by a constant n > 1 with its precomputed reciprocal (numerators below 2^16)
@@ -64,9 +74,16 @@ __device__ __forceinline__ Fix64 fix64(long long X) {
   const int lo = (int)(unsigned)X;
   return Fix64{lo, (int)(X >> 32) + (int)((unsigned)lo >> 31)};
 }
+// (sums modulo 2^64: where the total fits, partial sums may pass 2^63)
+__device__ __forceinline__ long long wrap_add(long long a, long long b) {
+  return (long long)((unsigned long long)a + (unsigned long long)b);
+}
+__device__ __forceinline__ long long wrap_sub(long long a, long long b) {
+  return (long long)((unsigned long long)a - (unsigned long long)b);
+}
 __device__ __forceinline__ void fix64_mac(long long& acc, int c, const Fix64& x) {
-  acc += (long long)c * (long long)x.lo;
-  acc += (long long)((unsigned long long)(unsigned)(c * x.hi) << 32);
+  acc = wrap_add(acc, (long long)c * (long long)x.lo);
+  acc = wrap_add(acc, (long long)((unsigned long long)((unsigned)c * (unsigned)x.hi) << 32));
 }
 
 // FP64 value of Y * 2^sh, rounded once to nearest: the two 32-bit halves as
@@ -82,13 +99,21 @@ __device__ __forceinline__ double fixed_rn(long long Y, int sh) {
 
 // The orbit operator of pattern P in 64-bit integers. Inputs are rounded to
 // the grid 2^(E + 1 - bits) (2^E the leading power of the group's largest
-// input), bits = 62 - log2 sum|a| (and 4 less for the transform of d = 4, whose
-// two butterflies grow the values by 16), so that every sum is exact in 64
-// bits; the only other rounding is the final one to FP64. Error: at most
-// sum|a| 2^(E - bits) + half a unit in the last place, below that of the FP64
-// sum (a rounding of every partial sum). Returns false for groups whose
-// exponents leave [emin, emax] (infinities and NaNs among them).
-template <int D, int P, class Sink>
+// input), bits = 62 - log2 sum|a| (d = 4: the largest for which four times the
+// result stays below 2^63), so that every sum is exact in 64 bits; the only other
+// rounding is the final one to FP64. Error: at most sum|a| 2^(E - bits) + half a unit
+// in the last place.
+// That is below the FP64 sum's (a rounding of every product and partial sum) where
+// an output takes the largest input of its group. An operator with zero coefficients
+// has outputs that take only some: where all of an output's inputs may lie far below
+// the largest (ka.below), the group is summed in FP64. Relative to sum |a x| of each
+// output, largest over 4000 random groups with magnitudes over 0 / 4 / 8 decades
+// (without that guard / with it / FP64 order): Table II row 2 1.1e-16, 3.2e-15, 8.1e-12 /
+// 1.1e-16, 1.4e-16, 2.1e-16 / 2.2e-16, 2.1e-16, 2.2e-16; row 5, whose outputs take all
+// inputs, 9e-17, 3e-16, 5e-16 / FP64 2.2e-16, 3.3e-16, 4.7e-16.
+// Returns false for such groups and for those whose exponents leave [emin, emax]
+// (infinities and NaNs among them).
+template <int D, int P, bool GUARD, class Sink>
 __device__ __forceinline__ bool fixed_sum(const KParams& kp, const KsArgs& ka, const double (&x)[Pat<D, P>::M],
                                           Sink&& sink) {
   constexpr int M = Pat<D, P>::M;
@@ -102,6 +127,17 @@ __device__ __forceinline__ bool fixed_sum(const KParams& kp, const KsArgs& ka, c
     for (int v = 0; v < M; v++) any |= (unsigned)__double2loint(x[v]);
     if (any != 0) return false;
     E = ka.emin;  // a group of zeros is exact on any grid
+  }
+  if (GUARD && ka.supp[P] != 0) {
+    const unsigned small = E > ka.below ? E - ka.below : 0;
+    int n = 0, z = 0;  // small inputs, and zeros (exact on any grid)
+#pragma unroll
+    for (int v = 0; v < M; v++) {
+      const unsigned a = (unsigned)__double2hiint(x[v]) & 0x7FFFFFFFu;
+      n += a < small;
+      z += (a | (unsigned)__double2loint(x[v])) == 0;
+    }
+    if (n > z && n >= ka.supp[P]) return false;
   }
   // (E | 0xFFFFF) - |x|'s high word borrows nothing from the exponent field
   const unsigned base = (E | 0xFFFFFu) + ((unsigned)(62 - ka.bits) << 20);
@@ -123,11 +159,11 @@ __device__ __forceinline__ bool fixed_sum(const KParams& kp, const KsArgs& ka, c
     for (int o = 0; o < NB; o++) {
       const long long x0 = X[kWht<P>.orb[o][0]], x1 = X[kWht<P>.orb[o][1]], x2 = X[kWht<P>.orb[o][2]],
                       x3 = X[kWht<P>.orb[o][3]];
-      const long long a0 = x0 + x1, a1 = x0 - x1, a2 = x2 + x3, a3 = x2 - x3;
-      t[4 * o] = fix64(a0 + a2);  // characters 0..3
-      t[4 * o + 1] = fix64(a1 + a3);
-      t[4 * o + 2] = fix64(a0 - a2);
-      t[4 * o + 3] = fix64(a1 - a3);
+      const long long a0 = x0 + x1, a1 = x0 - x1, a2 = x2 + x3, a3 = x2 - x3;  // below 2^62
+      t[4 * o] = fix64(wrap_add(a0, a2));  // characters 0..3
+      t[4 * o + 1] = fix64(wrap_add(a1, a3));
+      t[4 * o + 2] = fix64(wrap_sub(a0, a2));
+      t[4 * o + 3] = fix64(wrap_sub(a1, a3));
     }
 #pragma unroll
     for (int o = 0; o < NB; o++) {
@@ -139,8 +175,9 @@ __device__ __forceinline__ bool fixed_sum(const KParams& kp, const KsArgs& ka, c
         for (int q = 0; q < 6; q++)
           if (q < kWht<P>.nnz[i]) fix64_mac(yh[k], kp.wh[WOFF + kWht<P>.woff[i] + q], t[kWht<P>.col[i][q]]);
       }
-      const long long b0 = yh[0] + yh[1], b1 = yh[0] - yh[1], b2 = yh[2] + yh[3], b3 = yh[2] - yh[3];
-      const long long y4[4] = {b0 + b2, b1 + b3, b0 - b2, b1 - b3};  // 4 Y
+      const long long b0 = wrap_add(yh[0], yh[1]), b1 = wrap_sub(yh[0], yh[1]);
+      const long long b2 = wrap_add(yh[2], yh[3]), b3 = wrap_sub(yh[2], yh[3]);
+      const long long y4[4] = {wrap_add(b0, b2), wrap_add(b1, b3), wrap_sub(b0, b2), wrap_sub(b1, b3)};  // 4 Y
 #pragma unroll
       for (int vi = 0; vi < 4; vi++) sink(kWht<P>.orb[o][vi], fixed_rn(y4[vi], sh - 2));
     }
@@ -216,12 +253,12 @@ __device__ __forceinline__ void ks_group(const KParams& kp, const KsArgs& ka, un
     T x[M];
 #pragma unroll
     for (int u = 0; u < M; u++) x[u] = sm[ks_slot<D, P>(ka, u, val)];
-    if constexpr (AR == AR_FIXED || AR == AR_FIXED_MUL) {
+    if constexpr (AR == AR_FIXED || AR == AR_FIXED_MUL || AR == AR_FIXED_GUARD) {
       auto sink = [&](int u, double y) {
-        if constexpr (AR == AR_FIXED_MUL) y = __dmul_rn(kp.alpha, y);
+        if (AR == AR_FIXED_MUL || (AR == AR_FIXED_GUARD && D < 4 && (kp.flags & KF_ALPHA_MUL))) y = __dmul_rn(kp.alpha, y);
         sm[ks_slot<D, P>(ka, u, val)] = y;
       };
-      if (!fixed_sum<D, P>(kp, ka, x, sink)) ks_strict_group<D, P>(kp, ka, tup, sm);
+      if (!fixed_sum<D, P, AR == AR_FIXED_GUARD>(kp, ka, x, sink)) ks_strict_group<D, P>(kp, ka, tup, sm);
     } else {
       T y[M];
       apply_group<D, P, AR, T>(kp, x, y);
@@ -449,7 +486,8 @@ inline bool ks_plan(int d, const KParams& kp, int es, KsArgs* ka, int* smem, boo
   }
   int lg = 0;
   while ((double)(1 << lg) < L) lg++;
-  ka->bits = 62 - lg - (d == 4 ? 4 : 0);
+  // (d = 4: 4 L 2^bits < 2^63)
+  ka->bits = d == 4 ? ((double)(1 << lg) > L ? 61 - lg : 60 - lg) : 62 - lg;
   if (ka->bits > 60) ka->bits = 60;
   // kp.cexp = (53 - 2 W + kdrop + aexp) << 20 + 0x80000, aexp = alpha's and the coefficients' scale
   const int aexp = ((kp.cexp - 0x80000) >> 20) - 53 + 2 * kp.W - kp.kdrop;
@@ -462,6 +500,67 @@ inline bool ks_plan(int d, const KParams& kp, int es, KsArgs* ka, int* smem, boo
   ka->emin = (unsigned)lo << 20;
   ka->emax = (unsigned)hi << 20;
   return true;
+}
+
+// The inputs that the outputs of each pattern take, for fixed_sum's guard; *fixed is
+// cleared for operators whose outputs take so few that the guard would send groups
+// of like magnitudes to FP64 (of M uniform inputs, s or more lie 2^k below the largest
+// with a probability of about C(M, s) 2^(-(k + 1) s)).
+template <int D>
+void ks_support(const KParams& kp, KsArgs* ka, bool* fixed) {
+  static const Pattern<D> pt = make_pattern<D>(0);
+  static const std::array<int, 8> moff = [] {
+    std::array<int, 8> a{};
+    for (int p = 1; p < npatterns(D); p++) a[p] = mp_offset<D>(p);
+    return a;
+  }();
+  static const std::array<int, 8> mem = [] {
+    std::array<int, 8> a{};
+    for (int p = 0; p < npatterns(D); p++) a[p] = make_pattern<D>(p).m;
+    return a;
+  }();
+  constexpr int M = fact(D);
+  // the generic orbit: the chain's row of output 0, last stage first
+  double w[M] = {};
+  for (int s = 0; s < M; s++) w[pt.idx[0][s]] += kp.ci[kp.nci - 1][s];
+  for (int st = kp.nci - 2; st >= 0; st--) {
+    double t[M] = {};
+    for (int v = 0; v < M; v++)
+      for (int s = 0; s < M; s++) t[pt.idx[v][s]] += w[v] * kp.ci[st][s];
+    for (int v = 0; v < M; v++) w[v] = t[v];
+  }
+  int n = 0;
+  double sq = 0, least = 1e30;
+  for (double c : w)
+    if (c != 0) {
+      n++;
+      sq += c * c;
+      least = std::min(least, std::fabs(c));
+    }
+  for (int& v : ka->supp) v = 0;
+  ka->supp[0] = n < M ? n : 0;
+  bool any = ka->supp[0] != 0;
+  for (int p = 1; p < npatterns(D); p++) {
+    const int m = mem[p];
+    int few = m;
+    for (int u = 0; u < m; u++) {
+      int k = 0;
+      for (int v = 0; v < m; v++) k += kp.mp[moff[p] + u * m + v] != 0;
+      if (k > 0) few = std::min(few, k);
+    }
+    ka->supp[p] = few < m ? few : 0;
+    any = any || ka->supp[p] != 0;
+  }
+  if (!any || n == 0) return;
+  // an output's inputs reach 2^(E - k): the grid's share, about sqrt(sum a^2) 2^(E - bits), is
+  // then a few half units of the output's own sum
+  int k = (int)std::floor(ka->bits - 53 - std::log2(std::sqrt(sq) / least) + 2);
+  k = std::max(3, std::min(6, k));
+  ka->below = (unsigned)k << 20;
+  ka->guard = 1;
+  double few = 1;
+  for (int i = 0; i < ka->supp[0]; i++) few *= (double)(M - i) / (i + 1) / (2 << k);
+  if (ka->supp[0] != 0 && few > 0.002) *fixed = false;
 }
 
 // Whether KS is faster than KG, which takes a thread per orbit and position: a CTA of KS
@@ -521,15 +620,20 @@ bool launch_ks(const KParams& kp, int ar, cudaStream_t st, cudaError_t* e) {
   bool fixed = false;
   if (!ks_plan(D, kp, ar == AR_F32 ? 4 : 8, &ka, &smem, &fixed)) return false;
   fixed = fixed && ar == AR_EXACT;
+  if (fixed) ks_support<D>(kp, &ka, &fixed);
   if (!ks_faster(D, ar == AR_F32, fixed, kp.S, kp.O, ka.T)) return false;
   if constexpr (D == 4) {
     // 24-member groups take 128 registers: two CTAs of 256 threads, or, where a
     // block leaves room for one CTA only, one of 512
     if (ar == AR_F32) *e = launch_ks_impl<4, AR_F32, 256, 2, float>(kp, ka, smem, st);
-    else if (smem > KS_SMEM_MAX / 2) *e = launch_ks_impl<4, AR_FIXED, 512, 1, double>(kp, ka, smem, st);
+    else if (smem > KS_SMEM_MAX / 2)
+      *e = ka.guard ? launch_ks_impl<4, AR_FIXED_GUARD, 512, 1, double>(kp, ka, smem, st)
+                    : launch_ks_impl<4, AR_FIXED, 512, 1, double>(kp, ka, smem, st);
+    else if (ka.guard) *e = launch_ks_impl<4, AR_FIXED_GUARD, 256, 2, double>(kp, ka, smem, st);
     else *e = launch_ks_impl<4, AR_FIXED, 256, 2, double>(kp, ka, smem, st);
   } else {
     if (ar == AR_F32) *e = launch_ks_impl<D, AR_F32, 256, 5, float>(kp, ka, smem, st);
+    else if (fixed && ka.guard) *e = launch_ks_impl<D, AR_FIXED_GUARD, 256, 3, double>(kp, ka, smem, st);
     else if (fixed && (kp.flags & KF_ALPHA_MUL)) *e = launch_ks_impl<D, AR_FIXED_MUL, 256, 3, double>(kp, ka, smem, st);
     else if (fixed) *e = launch_ks_impl<D, AR_FIXED, 256, 3, double>(kp, ka, smem, st);
     else if constexpr (D == 2) *e = launch_ks_impl<D, AR_STRICT, 256, 3, double>(kp, ka, smem, st);
