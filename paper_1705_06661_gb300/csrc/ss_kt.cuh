@@ -85,7 +85,7 @@ struct KtShared {
   // matrix warp, and that at most two ahead of the epilogue
   unsigned rowexp[8][KT_ROWS];   // exponent fields
   unsigned colexp[16][KT_COLS];  // W's, by chunk mod 16 (the table warp runs ahead of the producers)
-  alignas(16) int tix[3][KT_CHUNK];  // tuple indices of a chunk (no tuple left: 0, and W's digits are 0)
+  alignas(16) int tix[3][KT_CHUNK];  // tuple indices of a chunk (no tuple left: another of the chunk's, and W's digits are 0)
   int pat[3][KT_UPC];            // pattern of each unit, -1: none
   int bad[8];                    // by tile mod 8: a scale is out of range
   uint64_t tab_full[3], tab_empty[3], mx_full[2], st_full[2], w_full[2], st_empty[2], acc_full[2], acc_empty[2], drain;
@@ -338,7 +338,8 @@ __device__ __forceinline__ int kt_members(int p) {
 // (Digitised by every row tile's CTA instead, W cost 0.16 of 0.56 ms on A[48^3,8^3].)
 template <int D>
 __global__ void __launch_bounds__(256) kt_prep_kernel(const __grid_constant__ KParams kp, const __grid_constant__ KtArgs ka) {
-  __shared__ int tix[KT_CHUNK];
+  __shared__ int tix[KT_CHUNK], tuples[KT_CHUNK];
+  __shared__ int wcount[KT_CHUNK / 32];
   __shared__ signed char none[KT_CHUNK];
   __shared__ unsigned colmax[KT_COLS];
   const int tid = threadIdx.x, ch = blockIdx.x, yt = blockIdx.y;
@@ -377,6 +378,25 @@ __global__ void __launch_bounds__(256) kt_prep_kernel(const __grid_constant__ KP
     }
     if (yt == 0 && o == 0) ka.pat[ch * KT_UPC + u] = p;
   }
+  __syncthreads();
+  // Slots without a tuple (their W is 0) repeat the chunk's own tuples in turn: the main
+  // kernel takes the chunk's row scales over all slots.
+  unsigned has = 0;
+  if (tid < KT_CHUNK) {
+    has = __ballot_sync(0xffffffffu, none[tid] == 0);
+    if ((tid & 31) == 0) wcount[tid >> 5] = __popc(has);
+  }
+  __syncthreads();
+  int ntup = 0, before = 0;  // tuples of the chunk, and of the slots before this one
+#pragma unroll
+  for (int w = 0; w < KT_CHUNK / 32; w++) {
+    if (w < tid >> 5) before += wcount[w];
+    ntup += wcount[w];
+  }
+  before += __popc(has & ((1u << (tid & 31)) - 1u));
+  if (tid < KT_CHUNK && none[tid] == 0) tuples[before] = tix[tid];
+  __syncthreads();
+  if (tid < KT_CHUNK && none[tid] != 0) tix[tid] = tuples[(tid - before) % ntup];
   __syncthreads();
   if (yt == 0 && tid < KT_CHUNK) ka.tix[ch * KT_CHUNK + tid] = tix[tid];
   const int y = tid & 31, q = tid >> 5;
