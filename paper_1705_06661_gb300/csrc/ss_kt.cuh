@@ -14,8 +14,8 @@
 //   column y of W each get one power-of-two scale (from the largest |A| resp. |W|
 //   of the chunk) and become 55-bit signed integers v = sum_i d_i 256^(6-i),
 //   i = 0..6, -128 <= d_i <= 127. The orbit operator runs on the integers of A
-//   (two limbs of 24 and up to 26 bits, 32-bit multiply-adds): S(A) is exact on
-//   the grid 2^(E + 1 - bits), bits = 54 - log2 sum|a|.
+//   (two limbs of 24 and up to 28 bits, 32-bit multiply-adds), rounded to the grid
+//   2^(E + 1 - bits), bits = 54 - log2 sum|a| and at most 52; S(A) is exact on it.
 // - D_d = sum over t and i + j = d of d_i(A) d_j(W), d = 0..6. Leading digits are at
 //   most 64, so |D_d| <= 192 d 2^14: below 2^24, hence exact in FP32, for d <= 5; D_6
 //   may round above 2^24, by a unit 2^-8 of the smallest that is kept.
@@ -130,20 +130,25 @@ __device__ __forceinline__ bool kt_sync(bool ok) {
   return r != 0;
 }
 
-// x on the grid of a scale as two limbs l1 2^24 + l0 of a signed integer, shifted up by
-// UP: the mantissa shifted right by (base - |x|'s high word) >> 20 places (base: the
-// scale's exponent field, plus the places that the grid drops, with 20 ones below it).
-// (One FP64 addition of 1.5 * 2^52 grid units does the same in five instructions, but at
-// two FP64 operations per SM and clock: 2509 against 2275 us on A[48^3,16^3].)
+// x rounded to the grid of a scale, as two limbs l1 2^24 + l0 of x's sign: the mantissa,
+// shifted up by UP, is shifted right to half grid units by (base - |x|'s high word) >> 20
+// places (base: the scale's exponent field, plus the places that the grid drops less
+// one, with 20 ones below it), and half of it plus one is the nearest integer, ties away
+// from zero. (Truncated instead, inputs of one sign lose half a unit each. The signs come
+// last, on the limbs: 2143 us on A[48^3,16^3] with 32 columns, as much as without
+// rounding; on the 64-bit integer before its rounding 2230. One FP64 addition of
+// 1.5 * 2^52 grid units does the same in five instructions, but at two FP64 operations
+// per SM and clock: 2509 against 2275 us there.)
 template <int UP>
 __device__ __forceinline__ void kt_limbs(double x, unsigned base, int& l0, int& l1) {
   const unsigned xh = (unsigned)__double2hiint(x), xl = (unsigned)__double2loint(x);
   const unsigned k = (base - (xh & 0x7FFFFFFFu)) >> 20;
-  const unsigned long long mant = ((unsigned long long)((xh & 0x000FFFFFu) | 0x00100000u) << 32) | xl;
+  const unsigned long long mant = (((unsigned long long)((xh & 0x000FFFFFu) | 0x00100000u) << 32) | xl) << UP;
   const long long q = (long long)shr64(mant, k);
-  const long long X = (int)xh < 0 ? -q : q;
-  l0 = (int)(((unsigned)X << UP) & 0xFFFFFFu);
-  l1 = (int)(X >> (24 - UP));
+  const unsigned long long r = (unsigned long long)q + 1;
+  const int sg = (int)xh >> 31;
+  l0 = (((int)((unsigned)(r >> 1) & 0xFFFFFFu)) ^ sg) - sg;
+  l1 = (((int)(r >> 25)) ^ sg) - sg;
 }
 
 // limbs y1 2^24 + y0 -> the biased digits: byte 3..0 of z1, then byte 2..0 of z0, each digit + 128
@@ -417,14 +422,14 @@ __global__ void __launch_bounds__(256) kt_prep_kernel(const __grid_constant__ KP
     E = KT_ELO;
   }
   if (q == 0) ka.wexp[((int64_t)yt * ka.nchunk + ch) * KT_COLS + y] = E | bad;
-  // largest |W| below 2^53, then shifted up by 1
+  // largest |W| at most 2^54
   const unsigned base = E | 0xFFFFFu;
   for (int kg = q; kg < KT_CHUNK / 8; kg += 8) {
     unsigned z0[8], z1[8];
 #pragma unroll
     for (int e = 0; e < 8; e++) {
       int l0, l1;
-      kt_limbs<1>(load(kg * 8 + e), base, l0, l1);
+      kt_limbs<2>(load(kg * 8 + e), base, l0, l1);
       kt_digits(l0, l1, z0[e], z1[e]);
     }
     unsigned char* dst = ka.wdig + (((int64_t)yt * ka.nchunk + ch) * 4 + kg / 6) * KT_WST + kg % 6 * KT_WKG + y * 16;
@@ -567,8 +572,8 @@ __global__ void __launch_bounds__(KT_THREADS, 1) kt_kernel(const __grid_constant
           E = KT_ELO;
         }
         if (half == 0) bad |= row < KT_COLS && sh.colexp[c & 15][row] >> 31;
-        // largest |A| below 2^bits
-        const unsigned base = (E + ((unsigned)(53 - ka.bits) << 20)) | 0xFFFFFu;
+        // largest |A| at most 2^bits
+        const unsigned base = (E + ((unsigned)(52 - ka.bits) << 20)) | 0xFFFFFu;
         const int ns = stages_of(ch);
         for (int j = 0; ok && j < ns; j++, n++) {
           if ((n & 1) != group) continue;  // the other group's stage
@@ -788,7 +793,7 @@ bool launch_kt(const KParams& kp, const double* W, int64_t Y, int64_t ldw, doubl
   ka.ldc = ldc;
   ka.ytiles = (int)((Y + KT_COLS - 1) / KT_COLS);
   ka.tiles = (kp.S + KT_ROWS - 1) / KT_ROWS * ka.ytiles;
-  ka.bits = lg > 0 ? 54 - lg : 53;  // a mantissa has 53 bits
+  ka.bits = lg > 2 ? 54 - lg : 52;  // (a mantissa has 53 bits, one of them for rounding)
   // kp.cexp = (53 - 2 W + kdrop + aexp) << 20 + 0x80000, aexp = the coefficients' scale;
   // a joined sum counts 2^56 of the products' units 2^(E_A + 1 - bits + aexp) 2^(E_W - 53)
   const int aexp = ((kp.cexp - 0x80000) >> 20) - 53 + 2 * kp.W - kp.kdrop;

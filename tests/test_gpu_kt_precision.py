@@ -1,6 +1,6 @@
 """What the tensor-core contraction's grids cost, against sums in extended
-precision: slots of a chunk that hold no tuple beside a very large element
-elsewhere."""
+precision: inputs of one sign (a truncated grid would bias them), and slots of a
+chunk that hold no tuple beside a very large element elsewhere."""
 import numpy as np
 import pytest
 
@@ -35,6 +35,22 @@ def _run(A, d, coef, W):
     C = ss.contract(a, coef, w, d=d, factorized=True)
     ss.spinsum_check_status(torch.cuda.current_stream().cuda_stream)
     return C.cpu().numpy().reshape(A.shape[0], W.shape[0])
+
+
+def test_inputs_of_one_sign_are_not_biased():
+    """Equal coefficients of 1-norm 126 leave 47 bits for A; every element in [1/2, 1) is rounded to 2^-47
+    independently, so an error beyond 8 standard deviations (and the one rounding of the only chunk) is a bias."""
+    d, O, S, Y = 3, 5, 400, 32
+    coef = np.full((1, 6), 21.0)
+    rng = np.random.default_rng(3)
+    A = 0.5 + 0.5 * rng.random((S,) + (O,) * d)
+    W = 0.5 + 0.5 * rng.random((Y,) + (O,) * d)
+    want = _flat(_summed(A, d, coef[0]), d) @ _flat(W, d).astype(np.longdouble).T
+    wsum = _flat(_summed(W, d, coef[0]), d)
+    sigma = 2.0 ** -47 / 12 ** 0.5 * np.sqrt((wsum ** 2).sum(axis=1))
+    err = np.abs(_run(A, d, coef, W) - want)
+    # W is rounded to 2^-54 or finer, and digit pairs below 2^-56 of the largest product are left out
+    assert np.all(err <= 8 * sigma + (2.0 ** -53 + 2.0 ** -51) * want)
 
 
 def test_empty_slots_do_not_coarsen_a_chunk():
