@@ -188,10 +188,12 @@ int spinsum_4d_host(int dtype, const int64_t ext[8], const void* A, const int64_
  * from 257 spectator positions on and where it is faster, the products run on
  * the tensor cores: S(A) and W as 55-bit integers on one power-of-two scale per
  * row resp. column and chunk of 192 tuples, every product and sum exact in
- * integers, one rounding to FP64 per chunk; tiles with infinities, NaN or
- * magnitudes beyond 2^+-440 are summed in FP64. Otherwise S(A) equals what
- * spinsum_3d/4d would store and is multiplied into FP64 accumulators in orbit
- * order. Either way |dC| <= (1e-14 + 2 O^d 2^-53) sum|a| max|A| max_y sum_t |W|.
+ * integers, one rounding to FP64 per chunk; tiles of 128 positions and 32
+ * columns with infinities, NaN or magnitudes beyond 2^+-440, or with magnitudes
+ * so far apart within a chunk that one scale would cost more bits than the FP64
+ * sums lose, take the FP64 form. There S(A) equals what spinsum_3d/4d would
+ * store and is multiplied into FP64 accumulators in orbit order, as it is with
+ * STRICT and for smaller calls. Either way |dC| <= (1e-14 + 2 O^d 2^-53) sum|a| max|A| max_y sum_t |W|.
  * The tensor-core path takes a stream-ordered workspace (W's digits, 448
  * bytes per tuple and 32 columns) from a pool of the library that keeps at
  * most 32 MB between calls; where none can be had the FP64 path runs. Under

@@ -86,7 +86,10 @@ __device__ __forceinline__ void kc_pattern(const KParams& kp, const double* __re
 
 template <int D, int AR, int YT, bool SUM>
 __global__ void __launch_bounds__(KC_THREADS) kc_kernel(const __grid_constant__ KParams kp, const double* __restrict__ W,
-                                                        int64_t Y, int64_t ldw, double* __restrict__ C, int64_t ldc) {
+                                                        int64_t Y, int64_t ldw, double* __restrict__ C, int64_t ldc,
+                                                        const unsigned char* __restrict__ flag) {
+  // after the tensor-core kernel: only the tiles of 128 rows and 32 columns that it left
+  if (flag && !flag[(int64_t)blockIdx.x / (128 / KC_THREADS) * ((Y + 31) / 32) + (int64_t)blockIdx.y * YT / 32]) return;
   const int64_t s = (int64_t)blockIdx.x * KC_THREADS + threadIdx.x;
   const int64_t y0 = (int64_t)blockIdx.y * YT;
   const int ny = (int)min((int64_t)YT, Y - y0);
@@ -117,13 +120,13 @@ __global__ void __launch_bounds__(KC_THREADS) kc_kernel(const __grid_constant__ 
 // one y-tile width per launch: 4, 8, 16 or 32 columns of C per thread
 template <int D, int AR, bool SUM>
 cudaError_t launch_kc_impl(const KParams& kp, const double* W, int64_t Y, int64_t ldw, double* C, int64_t ldc,
-                           cudaStream_t st) {
+                           cudaStream_t st, const unsigned char* flag = nullptr) {
   const int yt = Y <= 4 ? 4 : (Y <= 8 ? 8 : (Y <= 16 || D == 4 ? 16 : 32));
   const dim3 grid((unsigned)((kp.S + KC_THREADS - 1) / KC_THREADS), (unsigned)((Y + yt - 1) / yt));
-  if (yt == 4) kc_kernel<D, AR, 4, SUM><<<grid, KC_THREADS, 0, st>>>(kp, W, Y, ldw, C, ldc);
-  else if (yt == 8) kc_kernel<D, AR, 8, SUM><<<grid, KC_THREADS, 0, st>>>(kp, W, Y, ldw, C, ldc);
-  else if (yt == 16) kc_kernel<D, AR, 16, SUM><<<grid, KC_THREADS, 0, st>>>(kp, W, Y, ldw, C, ldc);
-  else if constexpr (D < 4) kc_kernel<D, AR, 32, SUM><<<grid, KC_THREADS, 0, st>>>(kp, W, Y, ldw, C, ldc);
+  if (yt == 4) kc_kernel<D, AR, 4, SUM><<<grid, KC_THREADS, 0, st>>>(kp, W, Y, ldw, C, ldc, flag);
+  else if (yt == 8) kc_kernel<D, AR, 8, SUM><<<grid, KC_THREADS, 0, st>>>(kp, W, Y, ldw, C, ldc, flag);
+  else if (yt == 16) kc_kernel<D, AR, 16, SUM><<<grid, KC_THREADS, 0, st>>>(kp, W, Y, ldw, C, ldc, flag);
+  else if constexpr (D < 4) kc_kernel<D, AR, 32, SUM><<<grid, KC_THREADS, 0, st>>>(kp, W, Y, ldw, C, ldc, flag);
   return cudaGetLastError();
 }
 

@@ -25,7 +25,22 @@
 //   D_d 256^(5-d), and D_6 rounded to D_5's unit), scaled, rounded once to FP64 and
 //   added to the FP64 sum of the chunks.
 // - A tile whose chunk scales leave a safe exponent range (infinities, NaN,
-//   magnitudes beyond 2^+-440) is recomputed in FP64 by its epilogue warps.
+//   magnitudes beyond 2^+-440), or whose magnitudes are too far apart for one
+//   scale (below), is left to KC, which follows and takes those tiles only.
+//
+// One scale per row and chunk costs the elements far below it their low bits. The
+// error, relative to sum_t |S(A) W| as that of FP64 sums is, is about 2^(q - bits) over
+// the square root of the number of tuples, where 2^-q is the mean of |A W| against the
+// product of the two largest. By the inequality of the means q is at most
+// the mean of log2(max|A| / |A|) plus that of log2(max|W| / |W|), which take one sum of
+// exponents each; the limit for it is bits - 43, where the error meets that of KC's
+// FP64 sums of a few hundred tuples, and a fluctuation, 6 / sqrt(tuples). Row 1 of Table
+// II, 512 tuples, largest error relative to sum |S W| (KT / KC, and q): uniform 1e-16 /
+// 4e-16, 3.0; Gaussian 2e-16 / 6e-16, 5.1; A and W over one decade each, W large where A
+// is small, 4e-16 / 6e-16, 5.9; over two 2e-15 / 4e-16, 8.9; over four 1e-13, 15. (A zero
+// counts as an element at the limit: it is exact on any grid.) The sums of exponents and
+// KC's launch over no tiles cost 3 %: 2148 -> 2225 us on A[48^3,16^3] with 32 columns (with a
+// shift and an addition in place of the dot product 2430).
 //
 // A CTA owns 128 rows x 32 columns. Warps 0-15 find the scales (a first read of
 // the chunk's A, which also brings it into L2), sum the orbits and write the digits;
@@ -55,6 +70,7 @@ constexpr int KT_WKG = KT_ND * KT_COLS * 16;      // bytes of 8 tuples of all di
 constexpr int KT_WST = 6 * KT_WKG;                // bytes of a stage of W
 constexpr int KT_STAGE = KT_ND * KT_AD + KT_WST;
 constexpr unsigned KT_ELO = (1023u - 440u) << 20, KT_EHI = (1023u + 440u) << 20;
+constexpr int KT_ZERO = (1023 - 440) * 16;        // a zero beside an element in that range, in 16ths
 
 template <int N>
 struct KtInt {
@@ -72,22 +88,29 @@ struct KtArgs {
   int bits;            // |A| < 2^bits on its grid
   int sh0;             // exponent of a joined sum's unit, less the two scales' exponents
   int opow[4];
+  int kappa;           // limit of the mean logarithms' sum, in 16ths
   // prepared by kt_prep_kernel in the call's workspace
   unsigned char* wdig;  // digits of W by column tile, chunk and stage
-  unsigned* wexp;       // [column tile][chunk][32] scales; top bit: out of range
+  unsigned* wexp;       // [column tile][chunk][32] scales
+  int* room;            // [column tile][chunk] what is left of the limit for A; -1: a scale is out of range
   int* tix;             // [chunk][192] tuple indices
   int* pat;             // [chunk][8] unit patterns, -1: none
+  // written by kt_kernel
+  unsigned char* flag;  // [tile] 1: left to KC
 };
 
 struct KtShared {
-  unsigned short rowmax[4][4][KT_ROWS];  // by chunk mod 4 and quarter: exponent of the largest |A|
+  // by chunk mod 4 and quarter: exponent of the largest |A| and the next four bits; sum of
+  // log2(largest / |A|) over the quarter's 48 tuples, in 16ths
+  unsigned short rowmax[4][4][KT_ROWS], rowlog[4][4][KT_ROWS];
   // chunk scales by chunk mod 8: producers run at most two chunks ahead of the
   // matrix warp, and that at most two ahead of the epilogue
   unsigned rowexp[8][KT_ROWS];   // exponent fields
   unsigned colexp[16][KT_COLS];  // W's, by chunk mod 16 (the table warp runs ahead of the producers)
   alignas(16) int tix[3][KT_CHUNK];  // tuple indices of a chunk (no tuple left: another of the chunk's, and W's digits are 0)
   int pat[3][KT_UPC];            // pattern of each unit, -1: none
-  int bad[8];                    // by tile mod 8: a scale is out of range
+  int room[3];                   // of the limit
+  int bad[8];                    // by tile mod 8: left to KC
   uint64_t tab_full[3], tab_empty[3], mx_full[2], st_full[2], w_full[2], st_empty[2], acc_full[2], acc_empty[2], drain;
   uint32_t tmem;
 };
@@ -347,9 +370,10 @@ __global__ void __launch_bounds__(256) kt_prep_kernel(const __grid_constant__ KP
   __shared__ int wcount[KT_CHUNK / 32];
   __shared__ signed char none[KT_CHUNK];
   __shared__ unsigned colmax[KT_COLS];
+  __shared__ int collog[KT_COLS], colzero[KT_COLS];
   const int tid = threadIdx.x, ch = blockIdx.x, yt = blockIdx.y;
   const int nunit = ka.upre[npatterns(D)];
-  if (tid < KT_COLS) colmax[tid] = 0;
+  if (tid < KT_COLS) colmax[tid] = collog[tid] = colzero[tid] = 0;
   if (tid < KT_CHUNK) {
     tix[tid] = 0;
     none[tid] = -1;
@@ -409,19 +433,36 @@ __global__ void __launch_bounds__(256) kt_prep_kernel(const __grid_constant__ KP
   const double* Wy = ka.W + (int64_t)yt * KT_COLS + y;
   auto load = [&](int e) { return act && none[e] == 0 ? Wy[(int64_t)tix[e] * ka.ldw] : 0.0; };
   unsigned m = 0;
+  int logs = 0, zeros = 0;
   for (int e = q; e < KT_CHUNK; e += 8) {
+    if (none[e] != 0) continue;
     const double v = load(e);
-    m = max(m, ((unsigned)__double2hiint(v) & 0x7FFFFFFFu) | ((unsigned)__double2loint(v) != 0));
+    const unsigned h = (unsigned)__double2hiint(v) & 0x7FFFFFFFu;
+    m = max(m, h | ((unsigned)__double2loint(v) != 0));
+    logs += h >> 16;
+    zeros += h == 0;
   }
   atomicMax(&colmax[y], m);
+  atomicAdd(&collog[y], logs);
+  atomicAdd(&colzero[y], zeros);
   __syncthreads();
   m = colmax[y];
-  unsigned E = m & 0x7FF00000u, bad = 0;
+  unsigned E = m & 0x7FF00000u;
+  bool bad = false;
   if (E < KT_ELO || E > KT_EHI) {
-    bad = m != 0 ? 0x80000000u : 0;
+    bad = m != 0;
     E = KT_ELO;
   }
-  if (q == 0) ka.wexp[((int64_t)yt * ka.nchunk + ch) * KT_COLS + y] = E | bad;
+  if (q == 0) {
+    ka.wexp[((int64_t)yt * ka.nchunk + ch) * KT_COLS + y] = E;
+    // per tuple, over the 192 slots of the rows' sums (a column of zeros contributes exact zeros)
+    const int far = m == 0 ? 0 : (ntup - colzero[y]) * (int)(m >> 16) - collog[y] + ka.kappa * colzero[y];
+    const int worst = __reduce_max_sync(0xffffffffu, far);
+    const int lim = (int)(KT_CHUNK * ((float)ka.kappa + 96.0f * rsqrtf((float)ntup)));
+    const bool out = __any_sync(0xffffffffu, bad), any = __any_sync(0xffffffffu, m != 0);
+    if (y == 0)
+      ka.room[yt * ka.nchunk + ch] = out ? -1 : (any ? max(0, lim - (int)((int64_t)worst * KT_CHUNK / ntup)) : 0x7FFFFFFF);
+  }
   // largest |W| at most 2^54
   const unsigned base = E | 0xFFFFFu;
   for (int kg = q; kg < KT_CHUNK / 8; kg += 8) {
@@ -437,31 +478,6 @@ __global__ void __launch_bounds__(256) kt_prep_kernel(const __grid_constant__ KP
   }
 }
 
-// FP64 form of one tile (rare): a thread per row, KC's loop over the orbits
-template <int D>
-static __device__ __noinline__ void kt_tile_fp64(const KParams& kp, const KtArgs& ka, int64_t s, int64_t y0, int ny) {
-  const bool act = s < kp.S;
-  for (int yb = 0; yb < ny; yb += 4) {
-    const int n = min(4, ny - yb);
-    const double* Wt = ka.W + y0 + yb;
-    double acc[4] = {0.0, 0.0, 0.0, 0.0};
-    kc_pattern<D, 0, AR_EXACT, 4, true>(kp, Wt, ka.ldw, n, s, act, acc);
-    kc_pattern<D, 1, AR_EXACT, 4, true>(kp, Wt, ka.ldw, n, s, act, acc);
-    if constexpr (D >= 3) {
-      kc_pattern<D, 2, AR_EXACT, 4, true>(kp, Wt, ka.ldw, n, s, act, acc);
-      kc_pattern<D, 3, AR_EXACT, 4, true>(kp, Wt, ka.ldw, n, s, act, acc);
-    }
-    if constexpr (D == 4) {
-      kc_pattern<D, 4, AR_EXACT, 4, true>(kp, Wt, ka.ldw, n, s, act, acc);
-      kc_pattern<D, 5, AR_EXACT, 4, true>(kp, Wt, ka.ldw, n, s, act, acc);
-      kc_pattern<D, 6, AR_EXACT, 4, true>(kp, Wt, ka.ldw, n, s, act, acc);
-      kc_pattern<D, 7, AR_EXACT, 4, true>(kp, Wt, ka.ldw, n, s, act, acc);
-    }
-    if (act)
-      for (int j = 0; j < n; j++) ka.C[s + ka.ldc * (y0 + yb + j)] = acc[j];
-  }
-}
-
 // FP64 value of Y * 2^sh, rounded once to nearest: the two 32-bit halves as
 // FP64 numbers with offsets 2^84 and 2^52 (times 2^sh)
 __device__ __forceinline__ double kt_to_double(long long Y, int sh) {
@@ -470,6 +486,19 @@ __device__ __forceinline__ double kt_to_double(long long Y, int sh) {
   const double c = __hiloint2double(0x45300000 + s, (int)0x80100000u);  // 2^84 + 2^63 + 2^52
   const double l = __hiloint2double(0x43300000 + s, (int)(unsigned)Y);
   return __dadd_rn(__dsub_rn(h, c), l);
+}
+
+// sum of top - log2|A| in 16ths over N tuples with zeros among them (or magnitudes far out
+// of range), kappa for a zero; out of line, rare
+template <int N>
+static __device__ __noinline__ int kt_logs_zeros(const unsigned* hw, const int* te, int64_t S, int top, int kappa) {
+  int logs = 0;
+#pragma unroll 1
+  for (int e = 0; e < N; e++) {
+    const unsigned h = hw[2 * (int64_t)te[e] * S] & 0x7FFFFFFFu;
+    logs += h != 0 ? top - (int)(h >> 16) : kappa;
+  }
+  return logs;
 }
 
 template <int D>
@@ -524,6 +553,7 @@ __global__ void __launch_bounds__(KT_THREADS, 1) kt_kernel(const __grid_constant
       const int* tix = sh.tix[c % 3];
       const double* As = row_of(tile);
       unsigned mx = 0;
+      int far = 0, n = 0;  // sum of log2(mx / |A|) in 16ths, tuples in it
       // high words only (half the registers: 24 loads in flight)
       const unsigned* hw = reinterpret_cast<const unsigned*>(As) + 1;
 #pragma unroll 1
@@ -540,15 +570,28 @@ __global__ void __launch_bounds__(KT_THREADS, 1) kt_kernel(const __grid_constant
           v[e + 3] = hw[2 * (int64_t)t.w * kp.S];
         }
         unsigned m = 0;
+        int logs = 0;
 #pragma unroll
-        for (int e = 0; e < N; e++) m = max(m, v[e] & 0x7FFFFFFFu);
+        for (int e = 0; e < N; e++) {
+          const unsigned h = v[e] & 0x7FFFFFFFu;
+          m = max(m, h);
+          logs = (int)__dp2a_lo(h, 0x0100u, (unsigned)logs);  // + (h >> 16), in one instruction
+        }
         if (m == 0) {  // zeros, or magnitudes below 2^-1042: the latter are out of range
           for (int e = 0; e < N; e++) m |= hw[2 * (int64_t)te[e] * kp.S - 1] != 0;
+          far += N * ka.kappa;
+        } else {
+          const int top = (int)(m >> 16), was = (int)(mx >> 16);
+          logs = N * top - logs;
+          if (logs >= KT_ZERO) logs = kt_logs_zeros<N>(hw, te, kp.S, top, ka.kappa);
+          far += logs + (top > was ? n * (top - was) : N * (was - top));
+          n += N;
         }
         mx = max(mx, m);
       }
-      // exponents only; 1 (out of range) for subnormal maxima
-      sh.rowmax[c & 3][quarter][row] = (unsigned short)(mx >> 20 == 0 && mx != 0 ? 1 : mx >> 20);
+      // exponent 1 (out of range) for subnormal maxima
+      sh.rowmax[c & 3][quarter][row] = (unsigned short)(mx >> 20 == 0 && mx != 0 ? 16 : mx >> 16);
+      sh.rowlog[c & 3][quarter][row] = (unsigned short)min(far, 65535);
       mbar_arrive(&sh.mx_full[c & 1]);
       return true;
     };
@@ -565,13 +608,22 @@ __global__ void __launch_bounds__(KT_THREADS, 1) kt_kernel(const __grid_constant
         if (!ok) break;
         const int* tix = sh.tix[c % 3];
         const unsigned short* rm = &sh.rowmax[c & 3][0][row];
-        unsigned E = max(max(rm[0], rm[KT_ROWS]), max(rm[2 * KT_ROWS], rm[3 * KT_ROWS])) << 20;
+        const int top = max(max(rm[0], rm[KT_ROWS]), max(rm[2 * KT_ROWS], rm[3 * KT_ROWS]));
+        unsigned E = (unsigned)(top >> 4) << 20;
         bool bad = false;
         if (E < KT_ELO || E > KT_EHI) {
           bad = E != 0;
           E = KT_ELO;
         }
-        if (half == 0) bad |= row < KT_COLS && sh.colexp[c & 15][row] >> 31;
+        if (half == 0) {
+          const unsigned short* rl = &sh.rowlog[c & 3][0][row];
+          int far = 0;
+#pragma unroll
+          for (int k = 0; k < 4; k++)
+            far += rl[k * KT_ROWS] + (rm[k * KT_ROWS] != 0 ? KT_CHUNK / 4 * (top - rm[k * KT_ROWS]) : 0);
+          const int room = sh.room[c % 3];
+          bad |= room < 0 || (top != 0 && far > room);
+        }
         // largest |A| at most 2^bits
         const unsigned base = (E + ((unsigned)(52 - ka.bits) << 20)) | 0xFFFFFu;
         const int ns = stages_of(ch);
@@ -647,7 +699,7 @@ __global__ void __launch_bounds__(KT_THREADS, 1) kt_kernel(const __grid_constant
             V += (long long)v[2] * (1 << 24) + (long long)v[3] * (1 << 16);
             V += (long long)v[4] * 256 + (long long)(v[5] + ((v[6] + 128) >> 8));
             const double a = __hiloint2double((int)hi[y], (int)lo[y]) +
-                             kt_to_double(V, er + (int)((sh.colexp[c & 15][yb + y] & 0x7FF00000u) >> 20));
+                             kt_to_double(V, er + (int)(sh.colexp[c & 15][yb + y] >> 20));
             lo[y] = (unsigned)__double2loint(a);
             hi[y] = (unsigned)__double2hiint(a);
           }
@@ -666,9 +718,9 @@ __global__ void __launch_bounds__(KT_THREADS, 1) kt_kernel(const __grid_constant
       }
       ok = kt_sync<2, 128>(ok);
       if (!ok) break;
-      if (bad) {
-        if (row == 0) sh.bad[it & 7] = 0;
-        kt_tile_fp64<D>(kp, ka, s, y0, ny);
+      if (row == 0) {
+        ka.flag[tile] = bad;
+        if (bad) sh.bad[it & 7] = 0;
       }
     }
   } else if (warp == MMA_WARP) {
@@ -724,6 +776,7 @@ __global__ void __launch_bounds__(KT_THREADS, 1) kt_kernel(const __grid_constant
             asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(a), "r"(bytes) : "memory");
         }
         if (lane < KT_UPC) sh.pat[c % 3][lane] = ka.pat[ch * KT_UPC + lane];
+        if (lane == 0) sh.room[c % 3] = ka.room[tile % ka.ytiles * ka.nchunk + ch];
         sh.colexp[c & 15][lane] = ka.wexp[(tile % ka.ytiles * ka.nchunk + ch) * KT_COLS + lane];
         mbar_arrive(&sh.tab_full[c % 3]);
       }
@@ -797,6 +850,7 @@ bool launch_kt(const KParams& kp, const double* W, int64_t Y, int64_t ldw, doubl
   // kp.cexp = (53 - 2 W + kdrop + aexp) << 20 + 0x80000, aexp = the coefficients' scale;
   // a joined sum counts 2^56 of the products' units 2^(E_A + 1 - bits + aexp) 2^(E_W - 53)
   const int aexp = ((kp.cexp - 0x80000) >> 20) - 53 + 2 * kp.W - kp.kdrop;
+  ka.kappa = 16 * (ka.bits - 43);
   ka.sh0 = 56 + 1 - ka.bits + aexp - 53 - 2 * 1023;
   if (aexp < -50 || aexp > 50) return false;
   int64_t units = 0;
@@ -833,18 +887,20 @@ bool launch_kt(const KParams& kp, const double* W, int64_t Y, int64_t ldw, doubl
   // workspace: the digits, scales and tuples; stream-ordered, so that calls on different
   // streams and threads have their own and nothing outlives the call
   const int64_t nd = (int64_t)ka.ytiles * ka.nchunk;
-  const int64_t bw = nd * 4 * KT_WST, be = nd * KT_COLS * 4, bt = (int64_t)ka.nchunk * KT_CHUNK * 4,
+  const int64_t bw = nd * 4 * KT_WST, be = nd * KT_COLS * 4, br = nd * 4, bt = (int64_t)ka.nchunk * KT_CHUNK * 4,
                 bp = (int64_t)ka.nchunk * KT_UPC * 4;
   unsigned char* ws = nullptr;
   cudaMemPool_t pool = kt_pool(dev);
-  if (!pool || ka.ytiles > 65535 || bw > (2LL << 30) || cudaMallocFromPoolAsync((void**)&ws, (size_t)(bw + be + bt + bp), pool, st) != cudaSuccess) {
+  if (!pool || ka.ytiles > 65535 || bw > (2LL << 30) || cudaMallocFromPoolAsync((void**)&ws, (size_t)(bw + be + br + bt + bp + ka.tiles), pool, st) != cudaSuccess) {
     cudaGetLastError();
     return false;  // KC needs no workspace
   }
   ka.wdig = ws;
   ka.wexp = reinterpret_cast<unsigned*>(ws + bw);
-  ka.tix = reinterpret_cast<int*>(ws + bw + be);
-  ka.pat = reinterpret_cast<int*>(ws + bw + be + bt);
+  ka.room = reinterpret_cast<int*>(ws + bw + be);
+  ka.tix = reinterpret_cast<int*>(ws + bw + be + br);
+  ka.pat = reinterpret_cast<int*>(ws + bw + be + br + bt);
+  ka.flag = ws + bw + be + br + bt + bp;
   const int64_t grid = ka.tiles < sms ? ka.tiles : sms;
   kt_prep_kernel<D><<<dim3((unsigned)ka.nchunk, (unsigned)ka.ytiles), 256, 0, st>>>(kp, ka);
   *e = cudaGetLastError();
@@ -852,6 +908,7 @@ bool launch_kt(const KParams& kp, const double* W, int64_t Y, int64_t ldw, doubl
     kt_kernel<D><<<(unsigned)grid, KT_THREADS, 2 * KT_STAGE, st>>>(kp, ka);
     *e = cudaGetLastError();
   }
+  if (*e == cudaSuccess) *e = launch_kc_impl<D, AR_EXACT, true>(kp, W, Y, ldw, C, ldc, st, ka.flag);
   const cudaError_t f = cudaFreeAsync(ws, st);
   if (*e == cudaSuccess) *e = f;
   return true;
