@@ -70,6 +70,7 @@ constexpr int KT_WKG = KT_ND * KT_COLS * 16;      // bytes of 8 tuples of all di
 constexpr int KT_WST = 6 * KT_WKG;                // bytes of a stage of W
 constexpr int KT_STAGE = KT_ND * KT_AD + KT_WST;
 constexpr unsigned KT_ELO = (1023u - 440u) << 20, KT_EHI = (1023u + 440u) << 20;
+constexpr int KT_VOTE = 4096;                     // most column tiles of a call that may be left to KC as a whole
 constexpr int KT_ZERO = (1023 - 440) * 16;        // a zero beside an element in that range, in 16ths
 
 template <int N>
@@ -93,6 +94,7 @@ struct KtArgs {
   unsigned char* wdig;  // digits of W by column tile, chunk and stage
   unsigned* wexp;       // [column tile][chunk][32] scales
   int* room;            // [column tile][chunk] what is left of the limit for A; -1: a scale is out of range
+  unsigned* vote;       // [column tile][chunk] which of eight sampled rows would be left to KC
   int* tix;             // [chunk][192] tuple indices
   int* pat;             // [chunk][8] unit patterns, -1: none
   // written by kt_kernel
@@ -371,6 +373,8 @@ __global__ void __launch_bounds__(256) kt_prep_kernel(const __grid_constant__ KP
   __shared__ signed char none[KT_CHUNK];
   __shared__ unsigned colmax[KT_COLS];
   __shared__ int collog[KT_COLS], colzero[KT_COLS];
+  __shared__ int left;
+  __shared__ unsigned votes;
   const int tid = threadIdx.x, ch = blockIdx.x, yt = blockIdx.y;
   const int nunit = ka.upre[npatterns(D)];
   if (tid < KT_COLS) colmax[tid] = collog[tid] = colzero[tid] = 0;
@@ -460,9 +464,35 @@ __global__ void __launch_bounds__(256) kt_prep_kernel(const __grid_constant__ KP
     const int worst = __reduce_max_sync(0xffffffffu, far);
     const int lim = (int)(KT_CHUNK * ((float)ka.kappa + 96.0f * rsqrtf((float)ntup)));
     const bool out = __any_sync(0xffffffffu, bad), any = __any_sync(0xffffffffu, m != 0);
-    if (y == 0)
-      ka.room[yt * ka.nchunk + ch] = out ? -1 : (any ? max(0, lim - (int)((int64_t)worst * KT_CHUNK / ntup)) : 0x7FFFFFFF);
+    if (y == 0) {
+      left = out ? -1 : (any ? max(0, lim - (int)((int64_t)worst * KT_CHUNK / ntup)) : 0x7FFFFFFF);
+      votes = 0;
+      ka.room[yt * ka.nchunk + ch] = left;
+    }
   }
+  __syncthreads();
+  // a warp per sampled row: the main kernel's rule
+  {
+    const double* As = static_cast<const double*>(kp.A) + (2 * q + 1) * kp.S / 16;
+    unsigned h[KT_CHUNK / 32], top = 0;
+    bool tiny = false;
+#pragma unroll
+    for (int e = 0; e < KT_CHUNK / 32; e++) {
+      const double v = As[(int64_t)tix[e * 32 + y] * kp.S];
+      h[e] = (unsigned)__double2hiint(v) & 0x7FFFFFFFu;
+      tiny |= h[e] == 0 && __double2loint(v) != 0;
+      top = max(top, h[e]);
+    }
+    top = __reduce_max_sync(0xffffffffu, top);
+    int far = 0;
+#pragma unroll
+    for (int e = 0; e < KT_CHUNK / 32; e++) far += h[e] != 0 ? (int)(top >> 16) - (int)(h[e] >> 16) : ka.kappa;
+    far = __reduce_add_sync(0xffffffffu, far);
+    const bool out = top == 0 ? __any_sync(0xffffffffu, tiny) : (top & 0x7FF00000u) < KT_ELO || (top & 0x7FF00000u) > KT_EHI;
+    if (y == 0 && (left < 0 || out || (top != 0 && far > left))) atomicOr(&votes, 1u << q);
+  }
+  __syncthreads();
+  if (tid == 0) ka.vote[yt * ka.nchunk + ch] = votes;
   // largest |W| at most 2^54
   const unsigned base = E | 0xFFFFFu;
   for (int kg = q; kg < KT_CHUNK / 8; kg += 8) {
@@ -501,11 +531,33 @@ static __device__ __noinline__ int kt_logs_zeros(const unsigned* hw, const int* 
   return logs;
 }
 
+// Where half the sampled rows of every column tile would be left to KC, the call is left to
+// it as a whole: inputs of spread magnitudes, or an infinity in W, would take both kernels'
+// time otherwise (25.7 against 27.9 ms on A[48^3,16^3] with 32 columns, 3.5 against 5.7 with
+// 4). Out of line, where it leaves the main kernel's code as it was (2231 us on ordinary
+// inputs; inlined 2480, and with the column tiles left out skipped one by one 2375).
+static __device__ __noinline__ bool kt_all_left(const KtArgs& ka, unsigned* votes) {
+  const int tid = threadIdx.x;
+  for (int i = tid; i < ka.ytiles; i += KT_THREADS) votes[i] = 0;
+  __syncthreads();
+  for (int i = tid; i < ka.ytiles * ka.nchunk; i += KT_THREADS)
+    if (const unsigned v = ka.vote[i]) atomicOr(&votes[i / ka.nchunk], v);
+  __syncthreads();
+  bool all = true;
+  for (int i = tid; i < ka.ytiles; i += KT_THREADS) all = all && __popc(votes[i]) >= 4;
+  all = __syncthreads_and(all);
+  if (all)
+    for (int64_t tile = blockIdx.x + (int64_t)tid * gridDim.x; tile < ka.tiles; tile += (int64_t)KT_THREADS * gridDim.x)
+      ka.flag[tile] = 1;
+  return all;
+}
+
 template <int D>
 __global__ void __launch_bounds__(KT_THREADS, 1) kt_kernel(const __grid_constant__ KParams kp, const __grid_constant__ KtArgs ka) {
   extern __shared__ __align__(128) unsigned char kt_smem[];
   __shared__ KtShared sh;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  if (ka.ytiles <= KT_VOTE && kt_all_left(ka, reinterpret_cast<unsigned*>(kt_smem))) return;
   if (tid == 0) {
     for (int i = 0; i < 3; i++) {
       mbar_init(&sh.tab_full[i], 32);
@@ -887,7 +939,7 @@ bool launch_kt(const KParams& kp, const double* W, int64_t Y, int64_t ldw, doubl
   // workspace: the digits, scales and tuples; stream-ordered, so that calls on different
   // streams and threads have their own and nothing outlives the call
   const int64_t nd = (int64_t)ka.ytiles * ka.nchunk;
-  const int64_t bw = nd * 4 * KT_WST, be = nd * KT_COLS * 4, br = nd * 4, bt = (int64_t)ka.nchunk * KT_CHUNK * 4,
+  const int64_t bw = nd * 4 * KT_WST, be = nd * KT_COLS * 4, br = nd * 8, bt = (int64_t)ka.nchunk * KT_CHUNK * 4,
                 bp = (int64_t)ka.nchunk * KT_UPC * 4;
   unsigned char* ws = nullptr;
   cudaMemPool_t pool = kt_pool(dev);
@@ -898,6 +950,7 @@ bool launch_kt(const KParams& kp, const double* W, int64_t Y, int64_t ldw, doubl
   ka.wdig = ws;
   ka.wexp = reinterpret_cast<unsigned*>(ws + bw);
   ka.room = reinterpret_cast<int*>(ws + bw + be);
+  ka.vote = reinterpret_cast<unsigned*>(ka.room + nd);
   ka.tix = reinterpret_cast<int*>(ws + bw + be + br);
   ka.pat = reinterpret_cast<int*>(ws + bw + be + br + bt);
   ka.flag = ws + bw + be + br + bt + bp;
