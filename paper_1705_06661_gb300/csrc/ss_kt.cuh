@@ -436,8 +436,14 @@ __global__ void __launch_bounds__(256) kt_prep_kernel(const __grid_constant__ KP
   const bool act = (int64_t)yt * KT_COLS + y < ka.Y;
   const double* Wy = ka.W + (int64_t)yt * KT_COLS + y;
   auto load = [&](int e) { return act && none[e] == 0 ? Wy[(int64_t)tix[e] * ka.ldw] : 0.0; };
+  // this warp's sampled row of A, for the votes below (loaded under the work on W)
+  double sample[KT_CHUNK / 32];
+#pragma unroll
+  for (int e = 0; e < KT_CHUNK / 32; e++)
+    sample[e] = static_cast<const double*>(kp.A)[(2 * q + 1) * kp.S / 16 + (int64_t)tix[e * 32 + y] * kp.S];
   unsigned m = 0;
   int logs = 0, zeros = 0;
+#pragma unroll 8
   for (int e = q; e < KT_CHUNK; e += 8) {
     if (none[e] != 0) continue;
     const double v = load(e);
@@ -473,14 +479,12 @@ __global__ void __launch_bounds__(256) kt_prep_kernel(const __grid_constant__ KP
   __syncthreads();
   // a warp per sampled row: the main kernel's rule
   {
-    const double* As = static_cast<const double*>(kp.A) + (2 * q + 1) * kp.S / 16;
     unsigned h[KT_CHUNK / 32], top = 0;
     bool tiny = false;
 #pragma unroll
     for (int e = 0; e < KT_CHUNK / 32; e++) {
-      const double v = As[(int64_t)tix[e * 32 + y] * kp.S];
-      h[e] = (unsigned)__double2hiint(v) & 0x7FFFFFFFu;
-      tiny |= h[e] == 0 && __double2loint(v) != 0;
+      h[e] = (unsigned)__double2hiint(sample[e]) & 0x7FFFFFFFu;
+      tiny |= h[e] == 0 && __double2loint(sample[e]) != 0;
       top = max(top, h[e]);
     }
     top = __reduce_max_sync(0xffffffffu, top);
