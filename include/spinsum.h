@@ -195,8 +195,9 @@ int spinsum_4d_host(int dtype, const int64_t ext[8], const void* A, const int64_
  * store and is multiplied into FP64 accumulators in orbit order, as it is with
  * STRICT and for smaller calls. Either way |dC| <= (1e-14 + 2 O^d 2^-53) sum|a| max|A| max_y sum_t |W|.
  * The tensor-core path takes a stream-ordered workspace (W's digits, 448
- * bytes per tuple and 32 columns) from a pool of the library that keeps at
- * most 32 MB between calls; where none can be had the FP64 path runs. Under
+ * bytes per tuple and 32 columns; where those exceed 128 MB, columns are taken
+ * in slabs as far as the positions allow, and none takes more than 2 GB) from a
+ * pool of the library that keeps at most 128 MB between calls; where none can be had the FP64 path runs. Under
  * stream capture the workspace becomes allocation and free nodes of the graph.
  * Errors: SPINSUM_ERR_ARG (bad d, extents,
  * leading dimensions, pointers or mode bits), SPINSUM_ERR_ALIAS (C overlaps A

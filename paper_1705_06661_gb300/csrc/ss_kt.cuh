@@ -53,6 +53,8 @@
 #include "ss_devcache.h"
 #include "ss_tma.cuh"
 
+#include <algorithm>
+
 #include <cuda_fp16.h>
 
 namespace ss {
@@ -844,7 +846,10 @@ __global__ void __launch_bounds__(KT_THREADS, 1) kt_kernel(const __grid_constant
   if (warp == MMA_WARP) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem));
 }
 
-// The library's memory pool for KT's workspaces on a device: freed blocks up to 32 MB
+// what the pool below keeps
+constexpr int64_t KT_POOL = 128 << 20;
+
+// The library's memory pool for KT's workspaces on a device: freed blocks up to 128 MB
 // stay with it between calls (the default pool would return them to the system at every
 // synchronisation and map them again, milliseconds). Null if the device has no pools.
 inline cudaMemPool_t kt_pool(int dev) {
@@ -859,7 +864,7 @@ inline cudaMemPool_t kt_pool(int dev) {
     cudaMemPool_t p = nullptr;
     cudaError_t err = cudaMemPoolCreate(&p, &props);
     if (err != cudaSuccess) return (int)err;
-    unsigned long long keep = 32ull << 20;
+    unsigned long long keep = KT_POOL;
     err = cudaMemPoolSetAttribute(p, cudaMemPoolAttrReleaseThreshold, &keep);
     *val = (long long)(uintptr_t)p;
     return (int)err;
@@ -895,9 +900,6 @@ bool launch_kt(const KParams& kp, const double* W, int64_t Y, int64_t ldw, doubl
   int lg = 0;
   while ((double)(1 << lg) < L) lg++;
   KtArgs ka{};
-  ka.W = W;
-  ka.C = C;
-  ka.Y = Y;
   ka.ldw = ldw;
   ka.ldc = ldc;
   ka.ytiles = (int)((Y + KT_COLS - 1) / KT_COLS);
@@ -941,13 +943,21 @@ bool launch_kt(const KParams& kp, const double* W, int64_t Y, int64_t ldw, doubl
     return true;
   }
   // workspace: the digits, scales and tuples; stream-ordered, so that calls on different
-  // streams and threads have their own and nothing outlives the call
-  const int64_t nd = (int64_t)ka.ytiles * ka.nchunk;
-  const int64_t bw = nd * 4 * KT_WST, be = nd * KT_COLS * 4, br = nd * 8, bt = (int64_t)ka.nchunk * KT_CHUNK * 4,
-                bp = (int64_t)ka.nchunk * KT_UPC * 4;
+  // streams and threads have their own and nothing outlives the call. A workspace above what
+  // the pool keeps is unmapped at the next synchronisation and mapped again by the next call
+  // (63 MB, A[300,30^3] with 133 columns, each call synchronised: 2436 us against 2199), so
+  // columns that need more are taken in slabs, as long as a slab gives every SM two tiles (in
+  // slabs of six tiles that call takes 6529 us).
+  const int64_t rows = ka.tiles / ka.ytiles, ytiles = ka.ytiles;
+  const int64_t bt = (int64_t)ka.nchunk * KT_CHUNK * 4, bp = (int64_t)ka.nchunk * KT_UPC * 4;
+  const int64_t per = (int64_t)ka.nchunk * (4 * KT_WST + KT_COLS * 4 + 8) + rows;  // of a column tile
+  const int64_t fit = std::min<int64_t>(32768, std::max<int64_t>((KT_POOL - bt - bp) / per, (2 * sms + rows - 1) / rows));
+  const int64_t nslab = (ka.ytiles + fit - 1) / fit, slab = (ka.ytiles + nslab - 1) / nslab;  // column tiles
+  const int64_t nd = slab * ka.nchunk, bw = nd * 4 * KT_WST, be = nd * KT_COLS * 4, br = nd * 8;
   unsigned char* ws = nullptr;
   cudaMemPool_t pool = kt_pool(dev);
-  if (!pool || ka.ytiles > 65535 || bw > (2LL << 30) || cudaMallocFromPoolAsync((void**)&ws, (size_t)(bw + be + br + bt + bp + ka.tiles), pool, st) != cudaSuccess) {
+  if (!pool || bw > (2LL << 30) ||
+      cudaMallocFromPoolAsync((void**)&ws, (size_t)(bw + be + br + bt + bp + slab * rows), pool, st) != cudaSuccess) {
     cudaGetLastError();
     return false;  // KC needs no workspace
   }
@@ -958,14 +968,22 @@ bool launch_kt(const KParams& kp, const double* W, int64_t Y, int64_t ldw, doubl
   ka.tix = reinterpret_cast<int*>(ws + bw + be + br);
   ka.pat = reinterpret_cast<int*>(ws + bw + be + br + bt);
   ka.flag = ws + bw + be + br + bt + bp;
-  const int64_t grid = ka.tiles < sms ? ka.tiles : sms;
-  kt_prep_kernel<D><<<dim3((unsigned)ka.nchunk, (unsigned)ka.ytiles), 256, 0, st>>>(kp, ka);
-  *e = cudaGetLastError();
-  if (*e == cudaSuccess) {
-    kt_kernel<D><<<(unsigned)grid, KT_THREADS, 2 * KT_STAGE, st>>>(kp, ka);
+  for (int64_t t0 = 0; t0 < ytiles && *e == cudaSuccess; t0 += slab) {
+    const int64_t y0 = t0 * KT_COLS;
+    ka.W = W + y0;
+    ka.C = C + ldc * y0;
+    ka.Y = std::min(Y - y0, slab * KT_COLS);
+    ka.ytiles = (int)((ka.Y + KT_COLS - 1) / KT_COLS);
+    ka.tiles = rows * ka.ytiles;
+    const int64_t grid = ka.tiles < sms ? ka.tiles : sms;
+    kt_prep_kernel<D><<<dim3((unsigned)ka.nchunk, (unsigned)ka.ytiles), 256, 0, st>>>(kp, ka);
     *e = cudaGetLastError();
+    if (*e == cudaSuccess) {
+      kt_kernel<D><<<(unsigned)grid, KT_THREADS, 2 * KT_STAGE, st>>>(kp, ka);
+      *e = cudaGetLastError();
+    }
+    if (*e == cudaSuccess) *e = launch_kc_impl<D, AR_EXACT, true>(kp, ka.W, ka.Y, ldw, ka.C, ldc, st, ka.flag);
   }
-  if (*e == cudaSuccess) *e = launch_kc_impl<D, AR_EXACT, true>(kp, W, Y, ldw, C, ldc, st, ka.flag);
   const cudaError_t f = cudaFreeAsync(ws, st);
   if (*e == cudaSuccess) *e = f;
   return true;

@@ -1,0 +1,51 @@
+"""The tensor-core contraction's workspace: columns in slabs that fit what the
+library's pool keeps."""
+import numpy as np
+import pytest
+
+import workloads as wl
+from tests.gpu_helpers import assert_bitexact
+
+pytestmark = pytest.mark.gpu
+
+
+def _place(x):
+    import torch
+    import paper_1705_06661_gb300 as ss
+    return ss.to_colmajor(torch.from_numpy(np.ascontiguousarray(x)).cuda())
+
+
+@pytest.mark.parametrize("d,O,S,Y", [(3, 30, 300, 133), (3, 16, 600, 2393)])
+def test_columns_in_slabs(d, O, S, Y):
+    """Many columns, at once and (75 columns of tiles, 70 at most) in slabs with a ragged last one; C
+    padded beyond S; integers are exact, the device's free memory moves by no more than what the pool keeps, and tiles left to the FP64
+    kernel (one row of spread magnitudes, an infinity in one column) are the right ones in every slab."""
+    import torch
+    import oracle
+    import paper_1705_06661_gb300 as ss
+    coef = wl.table2({3: 1, 4: 5}[d])
+    spec = (S,) + (1,) * (d - 1)
+    A, W = wl.integers(1, spec + (O,) * d), wl.integers(2, (Y, O ** d))
+    a, w = _place(A), _place(W)
+    base = torch.full(((S + 5) * Y,), 7.5, dtype=torch.float64, device="cuda")
+    out = base.as_strided(spec + (Y,), [1] + [S] * (d - 1) + [S + 5])
+    torch.cuda.synchronize()
+    ss.contract(a, coef, w, out=out, factorized=True)
+    torch.cuda.synchronize()
+    free0 = torch.cuda.mem_get_info()[0]
+    for _ in range(3):
+        ss.contract(a, coef, w, out=out, factorized=True)
+        torch.cuda.synchronize()
+        assert abs(torch.cuda.mem_get_info()[0] - free0) <= 2 << 20
+    ss.spinsum_check_status(torch.cuda.current_stream().cuda_stream)
+    want = oracle.contract(A, d, coef, W, factorized=True)
+    assert_bitexact(out.cpu().numpy(), want)
+    assert bool((base.view(Y, S + 5)[:, S:] == 7.5).all())
+    A[200] *= 2.0 ** -((np.arange(O ** d) % 40).reshape((1,) * (d - 1) + (O,) * d))
+    W[Y - 2, 3] = np.inf
+    with np.errstate(all="ignore"):
+        want = oracle.contract(A, d, coef, W, factorized=True)
+    got = ss.contract(_place(A), coef, _place(W), factorized=True).cpu().numpy()
+    keep = np.arange(S) != 200
+    assert_bitexact(got[keep], want[keep])
+    assert np.array_equal(np.isfinite(got), np.isfinite(want))
