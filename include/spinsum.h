@@ -28,7 +28,8 @@
  *
  * Ownership. The caller owns every buffer. A and B are device pointers; calls
  * are asynchronous on `stream` (a cudaStream_t; NULL = legacy default stream)
- * and allocate nothing. Coefficients, extents and strides are host memory,
+ * and allocate nothing (but for spinsum_plan_create, and spinsum_contract's
+ * workspace, see there). Coefficients, extents and strides are host memory,
  * read during the call only.
  *
  * Errors. Every entry point returns SPINSUM_OK (0) or a negative status and
@@ -197,8 +198,8 @@ int spinsum_4d_host(int dtype, const int64_t ext[8], const void* A, const int64_
  * The tensor-core path takes a stream-ordered workspace (W's digits, 448
  * bytes per tuple and 32 columns; where those exceed 128 MB, columns are taken
  * in slabs as far as the positions allow, and none takes more than 2 GB) from a
- * pool of the library that keeps at most 128 MB between calls; where none can be had the FP64 path runs. Under
- * stream capture the workspace becomes allocation and free nodes of the graph.
+ * pool of the library that keeps at most 128 MB between calls; where none can be had the FP64 path runs.
+ * Under stream capture the FP64 path runs too: the graph holds no allocation.
  * Errors: SPINSUM_ERR_ARG (bad d, extents,
  * leading dimensions, pointers or mode bits), SPINSUM_ERR_ALIAS (C overlaps A
  * or W), SPINSUM_ERR_CUDA. Asynchronous on `stream`.

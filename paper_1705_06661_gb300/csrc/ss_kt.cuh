@@ -862,7 +862,11 @@ inline cudaMemPool_t kt_pool(int dev) {
     props.location.type = cudaMemLocationTypeDevice;
     props.location.id = dev;
     cudaMemPool_t p = nullptr;
+    // (another thread may be capturing: creating a pool touches no stream)
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaThreadExchangeStreamCaptureMode(&mode);
     cudaError_t err = cudaMemPoolCreate(&p, &props);
+    cudaThreadExchangeStreamCaptureMode(&mode);
     if (err != cudaSuccess) return (int)err;
     unsigned long long keep = KT_POOL;
     err = cudaMemPoolSetAttribute(p, cudaMemPoolAttrReleaseThreshold, &keep);
@@ -923,6 +927,13 @@ bool launch_kt(const KParams& kp, const double* W, int64_t Y, int64_t ldw, doubl
   ka.nchunk = (int)((units + KT_UPC - 1) / KT_UPC);
   const int64_t ct = Y <= 4 ? 4 : (Y <= 8 ? 8 : (Y <= 16 || D == 4 ? 16 : 32)), kc_cols = (Y + ct - 1) / ct * ct;
   if (2.7 * KT_CHUNK * ka.nchunk * ka.ytiles > (double)T * kc_cols || (double)kp.S * T * kc_cols < 1e6) return false;
+  // A call under capture takes KC, which needs no workspace: one in the graph's own
+  // allocation nodes would keep the graph from being instantiated twice or put into another.
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+    cudaGetLastError();
+    return false;
+  }
   ka.opow[0] = 1;
   for (int k = 1; k < 4; k++) ka.opow[k] = k < D ? ka.opow[k - 1] * kp.O : 0;
   static DeviceCache cache;  // SMs, after raising the kernel's shared-memory limit

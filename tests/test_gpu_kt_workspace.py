@@ -49,3 +49,53 @@ def test_columns_in_slabs(d, O, S, Y):
     keep = np.arange(S) != 200
     assert_bitexact(got[keep], want[keep])
     assert np.array_equal(np.isfinite(got), np.isfinite(want))
+
+
+def test_captured_graph_holds_kernels_only():
+    """A captured call puts no allocation into the graph, so the graph can be instantiated twice, both
+    instances can run, and it can be a child of another graph."""
+    import ctypes
+    import torch
+    import oracle
+    import paper_1705_06661_gb300 as ss
+    cu = ctypes.CDLL("libcuda.so.1")
+
+    def ok(rc):
+        assert rc == 0, rc
+
+    d, O, S, Y = 3, 8, 400, 32
+    coef = wl.table2(1)
+    A, W = wl.integers(3, (S, 1, 1) + (O,) * d), wl.integers(4, (Y, O ** d))
+    want = oracle.contract(A, d, coef, W, factorized=True)
+    a, w, out = _place(A), _place(W), ss.colmajor_empty((S, 1, 1, Y))
+    ss.contract(a, coef, w, out=out, factorized=True)     # the tensor-core path
+    assert_bitexact(out.cpu().numpy(), want)
+    st = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    h = ctypes.c_void_p(st.cuda_stream)
+    ok(cu.cuStreamBeginCapture_v2(h, 0))
+    try:
+        ss.contract(a, coef, w, out=out, factorized=True, stream=st)
+    finally:
+        g = ctypes.c_void_p()
+        rc = cu.cuStreamEndCapture(h, ctypes.byref(g))
+    ok(rc)
+    n = ctypes.c_size_t(0)
+    ok(cu.cuGraphGetNodes(g, None, ctypes.byref(n)))
+    nodes = (ctypes.c_void_p * n.value)()
+    ok(cu.cuGraphGetNodes(g, nodes, ctypes.byref(n)))
+    for k in range(n.value):
+        t = ctypes.c_int(-1)
+        ok(cu.cuGraphNodeGetType(ctypes.c_void_p(nodes[k]), ctypes.byref(t)))
+        assert t.value == 0                               # a kernel
+    parent, child = ctypes.c_void_p(), ctypes.c_void_p()
+    ok(cu.cuGraphCreate(ctypes.byref(parent), 0))
+    ok(cu.cuGraphAddChildGraphNode(ctypes.byref(child), parent, None, ctypes.c_size_t(0), g))
+    for graph in (g, g, parent):
+        x = ctypes.c_void_p()
+        ok(cu.cuGraphInstantiateWithFlags(ctypes.byref(x), graph, ctypes.c_ulonglong(0)))
+        out.zero_()
+        torch.cuda.synchronize()
+        ok(cu.cuGraphLaunch(x, h))
+        torch.cuda.synchronize()
+        assert_bitexact(out.cpu().numpy(), want)
