@@ -27,6 +27,7 @@ cudaError_t launch_kc(int d, const KParams& kp, int ar, bool sum, const double* 
                       int64_t ldc, cudaStream_t st);
 int k1t_chunk(int d, int ar);
 
+void count_launches(int n);
 int* status_ptr();
 cudaError_t static_scratch_ptr(void** out);
 cudaError_t read_and_clear_status(int* out);
@@ -37,7 +38,12 @@ using namespace ss;
 namespace {
 
 thread_local std::string t_err;
-thread_local int64_t t_launches = 0;
+thread_local int64_t t_launches = 0;  // added to per launch_* call; more than one launch: count_launches
+
+}  // namespace
+// launches beyond the first of a launch_* call
+void ss::count_launches(int n) { t_launches += n; }
+namespace {
 
 int fail(int code, const char* fmt, ...) __attribute__((format(printf, 2, 3)));
 int fail(int code, const char* fmt, ...) {

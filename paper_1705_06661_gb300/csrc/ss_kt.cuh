@@ -59,6 +59,8 @@
 
 namespace ss {
 
+void count_launches(int n);
+
 constexpr int KT_ROWS = 128, KT_COLS = 32, KT_ND = 7;
 constexpr int KT_UNIT = 24;                       // tuples of a unit: 24 / m orbits of one pattern
 constexpr int KT_UPC = 8;                         // units of a chunk: four stages of two
@@ -995,6 +997,7 @@ bool launch_kt(const KParams& kp, const double* W, int64_t Y, int64_t ldw, doubl
     }
     if (*e == cudaSuccess) *e = launch_kc_impl<D, AR_EXACT, true>(kp, ka.W, ka.Y, ldw, ka.C, ldc, st, ka.flag);
   }
+  count_launches((int)(3 * nslab - 1));
   const cudaError_t f = cudaFreeAsync(ws, st);
   if (*e == cudaSuccess) *e = f;
   return true;

@@ -99,3 +99,18 @@ def test_captured_graph_holds_kernels_only():
         ok(cu.cuGraphLaunch(x, h))
         torch.cuda.synchronize()
         assert_bitexact(out.cpu().numpy(), want)
+
+
+def test_launches_are_counted():
+    """Three launches per slab on the tensor cores (digits of W, products, what is left to FP64), one on the
+    FP64 path."""
+    import torch
+    import paper_1705_06661_gb300 as ss
+    d, O, S = 3, 16, 600
+    coef, a = wl.table2(1), _place(wl.integers(5, (S, 1, 1) + (O,) * d))
+    for Y, strict, n in ((32, False, 3), (2393, False, 6), (32, True, 1)):
+        w = _place(wl.integers(6, (Y, O ** d)))
+        ss.spinsum_launch_count(reset=True)
+        ss.contract(a, coef, w, factorized=True, strict=strict)
+        assert ss.spinsum_launch_count(reset=True) == n
+    torch.cuda.synchronize()
