@@ -38,7 +38,7 @@ def to_colmajor(x: torch.Tensor) -> torch.Tensor:
 
 def _coef_chain(coef, d: int) -> np.ndarray:
     if type(coef) is np.ndarray and coef.ndim == 2 and coef.dtype == np.float64 and coef.flags.c_contiguous \
-            and coef.shape[1] == _FACT[d]:
+            and coef.shape[1] == math.factorial(d):
         return coef
     c = np.asarray(coef.detach().cpu().numpy() if isinstance(coef, torch.Tensor) else coef, dtype=np.float64)
     if c.ndim == 1:
@@ -46,9 +46,6 @@ def _coef_chain(coef, d: int) -> np.ndarray:
     if c.ndim != 2 or c.shape[1] != math.factorial(d):
         raise ValueError(f"coefficients must have shape [nfactors, {math.factorial(d)}]")
     return np.ascontiguousarray(c)
-
-
-_FACT = [math.factorial(k) for k in range(5)]
 
 
 # the current stream's handle without building a Stream object, where torch offers it
