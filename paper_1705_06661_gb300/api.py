@@ -55,7 +55,7 @@ _current_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None) or (
 
 def _raw_stream(stream, device: torch.device) -> int:
     """The CUDA stream handle to launch on: `stream`, or the device's current one."""
-    return _current_raw_stream(device.index) if stream is None else stream.cuda_stream
+    return stream.cuda_stream if stream else _current_raw_stream(device.index)
 
 
 def _dims(x: torch.Tensor, d: int):

@@ -20,3 +20,16 @@ def test_coefficients_of_any_dimension(api):
             api._coef_chain(np.ones((2, n + 1)), d)
     with pytest.raises(ValueError):
         api._coef_chain(np.ones((1, 24)), -1)
+
+
+def test_no_stream_means_the_current_one(api, monkeypatch):
+    """None and any other false value; elsewhere the API writes `stream or the current one`."""
+    import torch
+    monkeypatch.setattr(api, "_current_raw_stream", lambda index: 40 + index)
+    for none in (None, 0, False):
+        assert api._raw_stream(none, torch.device("cuda", 2)) == 42
+
+    class Stream:
+        cuda_stream = 7
+
+    assert api._raw_stream(Stream(), torch.device("cuda", 2)) == 7
