@@ -395,8 +395,13 @@ __global__ void __launch_bounds__(K2T_THREADS, MINB)
             k++;
         }
       }
-      // the answer is always waited for, so that none is in flight at the end
-      if (!__all_sync(0xffffffffu, mbar_wait(&sh.next_bar, ph, lim))) { ok = false; break; }
+      // the answer is always waited for, so that none is in flight at the end, also where the
+      // wait ran out (the block it may have taken over is then lost, and the call reported)
+      if (!__all_sync(0xffffffffu, mbar_wait(&sh.next_bar, ph, lim))) {
+        mbar_wait(&sh.next_bar, ph, kDrainLimit);
+        ok = false;
+        break;
+      }
       ph ^= 1;
       unsigned got = 0, x = 0;
       asm volatile(

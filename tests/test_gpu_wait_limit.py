@@ -58,3 +58,17 @@ def _run(body):
 
 def test_contraction():
     _run(CONTRACT)
+
+
+TILED = """
+for d, N in ((3, 96), (4, 28)):
+    A = wl.integers(d, (N,) * d)
+    coef_d = wl.table2({3: 1, 4: 5}[d])
+    a = ss.to_colmajor(torch.from_numpy(A).cuda())
+    b = ss.colmajor_like(a)
+    check(lambda: ss.spinsum(a, coef_d, d=d, out=b, factorized=True), lambda: b, oracle.spinsum(A, d, coef_d, factorized=True))
+"""
+
+
+def test_tiled_kernel():
+    _run(TILED)
