@@ -619,11 +619,12 @@ int run_pack(bool unpack, int d, int dtype, const int64_t* ext, const void* P, c
   return SPINSUM_OK;
 }
 
-int run(const Request& r, cudaStream_t st) {
+int run(const Request& r, cudaStream_t st, int flags = 0) {
   t_err.clear();
   Launch L;
   int rc = plan_one(r, &L);
   if (rc != SPINSUM_OK || L.empty) return rc;
+  L.kp.flags |= flags;
   L.kp.status = status_ptr();
   cudaError_t e = L.kernel == 0   ? launch_k1(r.d, L.kp, L.ar, L.vec, st)
                   : L.kernel == 2 ? launch_k1t(r.d, L.kp, L.ar, st)
@@ -820,7 +821,7 @@ int run_host(const Request& r, void* ws, size_t ws_bytes, cudaStream_t user) {
       Request q = r;
       q.A = pa.devicePointer;
       q.B = pb.devicePointer;
-      return run(q, user);
+      return run(q, user, KF_HOST);
     }
     cudaGetLastError();  // clear a sticky "invalid value" from probing pageable memory
   }

@@ -391,6 +391,7 @@ enum {
   KF_KDROP = 4,       // exact path: round the fixed-point sum before conversion
   KF_CHAIN = 16,      // K1, d <= 3: one of a plan's launches that may overlap (see launch_k1_bt)
   KF_CHAIN_NEXT = 32, // ... and not the first of them
+  KF_HOST = 64,       // A and B are host memory read and written over the link
   KF_WHT = 8,         // exact path, d = 4: freely transformable orbits through the Klein four-group transform
 };
 

@@ -26,8 +26,8 @@
 // block orbits leave room for four in flight per SM: the sums wait for loads).
 //
 // TMA needs 16-byte strides (even extents for FP64); other tensors, the beta
-// term, strict order, dense d = 4 operators and d = 2 (two 8 KB tiles per block
-// orbit: 271 us against K2's 217 at N = 8192) stay with K2.
+// term, strict order, dense d = 4 operators, tensors in host memory and d = 2 (two
+// 8 KB tiles per block orbit: 271 us against K2's 217 at N = 8192) stay with K2.
 #include <cuda.h>
 
 #include "ss_k2.cuh"
@@ -499,7 +499,7 @@ bool k2t_map(CUtensorMap* map, const void* p, const int64_t* ld, int64_t N) {
 // true (and *e the launch status) when K2T takes the problem
 template <int D, int AR, int NST, int MINB, typename T>
 bool launch_k2t(const KParams& kp, cudaStream_t st, cudaError_t* e) {
-  if (kp.flags & KF_BETA) return false;
+  if (kp.flags & (KF_BETA | KF_HOST)) return false;
   CUtensorMap ma, mb;
   if (!k2t_map<D, T>(&ma, kp.A, kp.lda, kp.O) || !k2t_map<D, T>(&mb, kp.B, kp.ldb, kp.O)) return false;
   auto fn = k2t_kernel<D, AR, NST, MINB, T>;
