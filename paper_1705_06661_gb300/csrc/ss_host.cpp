@@ -518,12 +518,25 @@ int plan_one(const Request& r, Launch* L) {
       // with the L2 prefetch of the next chunk)
       const int64_t pos = (d == 4 && (kp.flags & KF_WHT)) ? SS_K1_POS4 : 8192;
       int64_t cpb0 = std::min<int64_t>(kp.nchunk, std::max<int64_t>(1, pos / per));
-      // few orbits: enough blocks for about three rounds of the resident CTAs (O = 6 has 56
-      // orbits for d = 3; 336 blocks of 8192 positions left half the SMs idle)
+      // Few orbits leave SMs idle with blocks that long. A block costs its set-up (the search
+      // of its tuple: about as long as SETUP chunks) and its chunks; all blocks share the
+      // resident CTAs, and the last ones run out on their own. us per call with 1, 2, 4, .. chunks
+      // per block: A[8000,10^3] FP64 32.8, 30.6, 28.6, 44 (16); A[64000,6^3] 46.5 (3), 43.7 (4),
+      // 55 (16); A[4096,6^4] 31 (2), 28.6 (4), 37 (8), 66 (16); A[1000,10^4] 58 (1), 41.7 (4).
       int64_t orbits = 0;
       for (int p = 0; p < np; p++) orbits += kp.norb[p];
-      const int64_t min_bpo = (SS_K1_MINBLOCKS + orbits - 1) / std::max<int64_t>(orbits, 1);
-      cpb0 = std::min(cpb0, std::max<int64_t>(1, kp.nchunk / min_bpo));
+      const double setup = d == 4 ? 3.0 : 1.5, resident = 152.0 * (d == 4 ? 3 : 4);
+      double least = 1e300;
+      int64_t best = cpb0;
+      for (int64_t c = cpb0; c >= 1; c--) {
+        const double blocks = (double)orbits * ((kp.nchunk + c - 1) / c);
+        const double cost = (blocks / resident + 1.0) * (setup + (double)c);
+        if (cost < least) {
+          least = cost;
+          best = c;
+        }
+      }
+      cpb0 = best;
       const int64_t nbo = (kp.nchunk + cpb0 - 1) / cpb0;
       kp.cpb = (int)((kp.nchunk + nbo - 1) / nbo);
       const int64_t bpo = (kp.nchunk + kp.cpb - 1) / kp.cpb;

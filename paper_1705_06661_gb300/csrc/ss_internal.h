@@ -349,12 +349,6 @@ constexpr int MP_MAX = MP_TOTAL_4;
 #ifndef SS_K1_KB0F32
 #define SS_K1_KB0F32 2
 #endif
-// K1: blocks that a problem of few orbits is cut into (three rounds of four CTAs on 152 SMs;
-// two / three / four / eight rounds: 32 uneven 3D blocks chained 2969 / 2990 / 3055 / 3197 us,
-// 4D 10^8 forward and backward 578 / 571 / 571 / 599 us)
-#ifndef SS_K1_MINBLOCKS
-#define SS_K1_MINBLOCKS 1824
-#endif
 // K1, d = 4 transform path: spectator positions per member per block
 #ifndef SS_K1_POS4
 #define SS_K1_POS4 5120
