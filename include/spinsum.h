@@ -194,7 +194,8 @@ int spinsum_4d_host(int dtype, const int64_t ext[8], const void* A, const int64_
  * so far apart within a chunk that one scale would cost more bits than the FP64
  * sums lose, take the FP64 form. There S(A) equals what spinsum_3d/4d would
  * store and is multiplied into FP64 accumulators in orbit order, as it is with
- * STRICT and for smaller calls. Either way |dC| <= (1e-14 + 2 O^d 2^-53) sum|a| max|A| max_y sum_t |W|.
+ * STRICT and for smaller calls (so that such a call equals the summation stored
+ * by spinsum_3d/4d and then contracted, coef == NULL, bit for bit). Either way |dC| <= (1e-14 + 2 O^d 2^-53) sum|a| max|A| max_y sum_t |W|.
  * The tensor-core path takes a stream-ordered workspace (W's digits, 448
  * bytes per tuple and 32 columns; where those exceed 128 MB, columns are taken
  * in slabs as far as the positions allow, and none takes more than 2 GB) from a

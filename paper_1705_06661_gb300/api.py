@@ -120,7 +120,14 @@ def contract(A: torch.Tensor, coef, W: torch.Tensor, *, d: int | None = None, ou
     never stored (spinsum_contract); coef None contracts A itself. A: FP64,
     dense column-major (d spectators, d permuted indices). W: FP64, shape
     (Y, O**d), y fastest (a column-major copy is made otherwise). Returns C of
-    shape (spectators..., Y), column-major (a new tensor unless `out` is one)."""
+    shape (spectators..., Y), column-major (a new tensor unless `out` is one).
+
+    Calls of more than 256 spectator positions with integer coefficients run on
+    the tensor cores, S(A) and W as integers on one scale per row (column) and
+    192 tuples; where magnitudes are too far apart for that, under stream
+    capture and with strict=True they run in FP64. The bits of the result
+    depend on that choice (and so does their equality with the unfused pair of
+    calls); strict=True makes it, and takes no workspace."""
     if d is None:
         d = A.dim() // 2
     if A.dim() != 2 * d or A.dtype != torch.float64 or not A.is_cuda:

@@ -3,7 +3,7 @@
 
 namespace ss {
 
-// FP64: 24 KB stages, four per CTA and two CTAs per SM (A[544]^3: 426 us; three by three
+// FP64: 24 KB stages, four per CTA and two CTAs per SM (A[544]^3: 426 us at that time, 406 now; three by three
 // 448, two groups of eight warps on four stages 445, on nine stages of one CTA 641)
 bool launch_k2t_d3(const KParams& kp, int ar, cudaStream_t st, cudaError_t* e) {
   if (ar == AR_EXACT) return launch_k2t<3, AR_EXACT, 4, 2, double>(kp, st, e);

@@ -184,6 +184,17 @@ __device__ __forceinline__ bool exact_limbs(const KParams& kp, const double (&x)
   return true;
 }
 
+// FP64 value of Y * 2^sh, rounded once to nearest: the two 32-bit halves as
+// FP64 numbers with offsets 2^84 and 2^52 (times 2^sh); their difference to
+// the joint offset is exact and the last addition rounds.
+__device__ __forceinline__ double fixed_rn(long long Y, int sh) {
+  const int s = (int)((unsigned)sh << 20);
+  const double h = __hiloint2double(0x45300000 + s, (int)((unsigned)(Y >> 32) ^ 0x80000000u));
+  const double c = __hiloint2double(0x45300000 + s, (int)0x80100000u);  // 2^84 + 2^63 + 2^52
+  const double l = __hiloint2double(0x43300000 + s, (int)(unsigned)Y);
+  return __dadd_rn(__dsub_rn(h, c), l);
+}
+
 // limbs (y1 * 2^W + y0) -> FP64: round off kdrop bits on the low limb
 // ((y1 2^W + y0 + r) >> k = y1 2^(W-k) + ((y0 + r) >> k) for k <= W), then one
 // subtraction of the magic constant C = chi:0

@@ -86,17 +86,6 @@ __device__ __forceinline__ void fix64_mac(long long& acc, int c, const Fix64& x)
   acc = wrap_add(acc, (long long)((unsigned long long)((unsigned)c * (unsigned)x.hi) << 32));
 }
 
-// FP64 value of Y * 2^sh, rounded once to nearest: the two 32-bit halves as
-// FP64 numbers with offsets 2^84 and 2^52 (times 2^sh); their difference to
-// the joint offset is exact and the last addition rounds.
-__device__ __forceinline__ double fixed_rn(long long Y, int sh) {
-  const int s = (int)((unsigned)sh << 20);
-  const double h = __hiloint2double(0x45300000 + s, (int)((unsigned)(Y >> 32) ^ 0x80000000u));
-  const double c = __hiloint2double(0x45300000 + s, (int)0x80100000u);  // 2^84 + 2^63 + 2^52
-  const double l = __hiloint2double(0x43300000 + s, (int)(unsigned)Y);
-  return __dadd_rn(__dsub_rn(h, c), l);
-}
-
 // The orbit operator of pattern P in 64-bit integers. Inputs are rounded to
 // the grid 2^(E + 1 - bits) (2^E the leading power of the group's largest
 // input), bits = 62 - log2 sum|a| (d = 4: the largest for which four times the

@@ -77,11 +77,6 @@ constexpr unsigned KT_ELO = (1023u - 440u) << 20, KT_EHI = (1023u + 440u) << 20;
 constexpr int KT_VOTE = 4096;                     // most column tiles of a call that may be left to KC as a whole
 constexpr int KT_ZERO = (1023 - 440) * 16;        // a zero beside an element in that range, in 16ths
 
-template <int N>
-struct KtInt {
-  static constexpr int value = N;
-};
-
 struct KtArgs {
   const double* W;
   double* C;
@@ -228,7 +223,7 @@ __device__ __forceinline__ void kt_load(const double* As, int64_t S, const int* 
 // the wait and the choice of the pattern hide their latency: 2222 -> 2119 us on
 // A[48^3,16^3] with 32 columns; all 24 of them do not fit into 80 registers)
 template <int D, int P>
-__device__ __forceinline__ void kt_unit(const KParams& kp, const KtArgs& ka, const double* As, const int* tix,
+__device__ __forceinline__ void kt_unit(const KParams& kp, const double* As, const int* tix,
                                         unsigned base, unsigned char* dst, double (&x0)[12]) {
   constexpr int M = Pat<D, P>::M, NO = KT_UNIT / M;
   if constexpr (M == 24) {
@@ -325,17 +320,17 @@ __device__ __forceinline__ void kt_unit(const KParams& kp, const KtArgs& ka, con
 }
 
 template <int D>
-__device__ __forceinline__ void kt_unit_any(const KParams& kp, const KtArgs& ka, int p, const double* As,
+__device__ __forceinline__ void kt_unit_any(const KParams& kp, int p, const double* As,
                                             const int* tix, unsigned base, unsigned char* dst, double (&x0)[12]) {
   switch (p) {
-    case 0: kt_unit<D, 0>(kp, ka, As, tix, base, dst, x0); break;
-    case 1: kt_unit<D, 1>(kp, ka, As, tix, base, dst, x0); break;
-    case 2: if constexpr (npatterns(D) > 2) kt_unit<D, 2>(kp, ka, As, tix, base, dst, x0); break;
-    case 3: if constexpr (npatterns(D) > 3) kt_unit<D, 3>(kp, ka, As, tix, base, dst, x0); break;
-    case 4: if constexpr (npatterns(D) > 4) kt_unit<D, 4>(kp, ka, As, tix, base, dst, x0); break;
-    case 5: if constexpr (npatterns(D) > 4) kt_unit<D, 5>(kp, ka, As, tix, base, dst, x0); break;
-    case 6: if constexpr (npatterns(D) > 4) kt_unit<D, 6>(kp, ka, As, tix, base, dst, x0); break;
-    case 7: if constexpr (npatterns(D) > 4) kt_unit<D, 7>(kp, ka, As, tix, base, dst, x0); break;
+    case 0: kt_unit<D, 0>(kp, As, tix, base, dst, x0); break;
+    case 1: kt_unit<D, 1>(kp, As, tix, base, dst, x0); break;
+    case 2: if constexpr (npatterns(D) > 2) kt_unit<D, 2>(kp, As, tix, base, dst, x0); break;
+    case 3: if constexpr (npatterns(D) > 3) kt_unit<D, 3>(kp, As, tix, base, dst, x0); break;
+    case 4: if constexpr (npatterns(D) > 4) kt_unit<D, 4>(kp, As, tix, base, dst, x0); break;
+    case 5: if constexpr (npatterns(D) > 4) kt_unit<D, 5>(kp, As, tix, base, dst, x0); break;
+    case 6: if constexpr (npatterns(D) > 4) kt_unit<D, 6>(kp, As, tix, base, dst, x0); break;
+    case 7: if constexpr (npatterns(D) > 4) kt_unit<D, 7>(kp, As, tix, base, dst, x0); break;
     default:  // no tuples left: digits of zero
       const unsigned z[8] = {0x80808080u, 0x80808080u, 0x80808080u, 0x80808080u, 0x80808080u, 0x80808080u, 0x80808080u, 0x80808080u};
       for (int g = 0; g < 3; g++) kt_store8(dst + g * KT_AKG, KT_AD, z, z);
@@ -514,16 +509,6 @@ __global__ void __launch_bounds__(256) kt_prep_kernel(const __grid_constant__ KP
     unsigned char* dst = ka.wdig + (((int64_t)yt * ka.nchunk + ch) * 4 + kg / 6) * KT_WST + kg % 6 * KT_WKG + y * 16;
     kt_store8(dst, KT_COLS * 16, z0, z1);
   }
-}
-
-// FP64 value of Y * 2^sh, rounded once to nearest: the two 32-bit halves as
-// FP64 numbers with offsets 2^84 and 2^52 (times 2^sh)
-__device__ __forceinline__ double kt_to_double(long long Y, int sh) {
-  const int s = (int)((unsigned)sh << 20);
-  const double h = __hiloint2double(0x45300000 + s, (int)((unsigned)(Y >> 32) ^ 0x80000000u));
-  const double c = __hiloint2double(0x45300000 + s, (int)0x80100000u);  // 2^84 + 2^63 + 2^52
-  const double l = __hiloint2double(0x43300000 + s, (int)(unsigned)Y);
-  return __dadd_rn(__dsub_rn(h, c), l);
 }
 
 // sum of top - log2|A| in 16ths over N tuples with zeros among them (or magnitudes far out
@@ -709,7 +694,7 @@ __global__ void __launch_bounds__(KT_THREADS, 1) kt_kernel(const __grid_constant
             bulk_g2s(st + KT_ND * KT_AD, wd + ((int64_t)ch * 4 + j) * KT_WST, KT_WST, &sh.w_full[group]);
             copies++;
           }
-          kt_unit_any<D>(kp, ka, sh.pat[c % 3][u], As, tix + u * KT_UNIT, base, st + half * 3 * KT_AKG + row * 16, x0);
+          kt_unit_any<D>(kp, sh.pat[c % 3][u], As, tix + u * KT_UNIT, base, st + half * 3 * KT_AKG + row * 16, x0);
           kt_proxy_fence();
           mbar_arrive(&sh.st_full[n & 1]);
         }
@@ -759,7 +744,7 @@ __global__ void __launch_bounds__(KT_THREADS, 1) kt_kernel(const __grid_constant
             V += (long long)v[2] * (1 << 24) + (long long)v[3] * (1 << 16);
             V += (long long)v[4] * 256 + (long long)(v[5] + ((v[6] + 128) >> 8));
             const double a = __hiloint2double((int)hi[y], (int)lo[y]) +
-                             kt_to_double(V, er + (int)(sh.colexp[c & 15][yb + y] >> 20));
+                             fixed_rn(V, er + (int)(sh.colexp[c & 15][yb + y] >> 20));
             lo[y] = (unsigned)__double2loint(a);
             hi[y] = (unsigned)__double2hiint(a);
           }

@@ -145,3 +145,17 @@ def test_spread_rows_leave_the_others_alone():
     keep = np.r_[6:256, 384:S]
     assert np.array_equal(got[keep][:, :32], base[keep][:, :32]) and np.array_equal(got[keep][:, 64:], base[keep][:, 64:])
     assert not np.array_equal(got[:128, :32], pair[:128, :32])
+
+
+def test_strict_equals_the_unfused_pair():
+    """With STRICT a call of any size is FP64 throughout: that of the strict summation, stored and contracted."""
+    import torch
+    import paper_1705_06661_gb300 as ss
+    d, O, S, Y = 3, 8, 300, 32
+    A, W = _spread(d, O, S, Y, 0, False, 12)
+    a = ss.to_colmajor(torch.from_numpy(np.ascontiguousarray(A.reshape((S, 1, 1) + (O,) * d))).cuda())
+    w = ss.to_colmajor(torch.from_numpy(np.ascontiguousarray(_flat(W, d))).cuda())
+    coef = wl.table2(1)
+    got = ss.contract(a, coef, w, factorized=True, strict=True)
+    pair = ss.contract(ss.spinsum(a, coef, factorized=True, strict=True), None, w)
+    assert torch.equal(got, pair)
