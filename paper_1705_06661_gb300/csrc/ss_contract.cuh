@@ -88,7 +88,9 @@ template <int D, int AR, int YT, bool SUM>
 __global__ void __launch_bounds__(KC_THREADS) kc_kernel(const __grid_constant__ KParams kp, const double* __restrict__ W,
                                                         int64_t Y, int64_t ldw, double* __restrict__ C, int64_t ldc,
                                                         const unsigned char* __restrict__ flag) {
-  // after the tensor-core kernel: only the tiles of 128 rows and 32 columns that it left
+  // after the tensor-core kernel, under whose end it may be launched: only the tiles of 128 rows
+  // and 32 columns that it left
+  if (flag) asm volatile("griddepcontrol.wait;" ::: "memory");
   if (flag && !flag[(int64_t)blockIdx.x / (128 / KC_THREADS) * ((Y + 31) / 32) + (int64_t)blockIdx.y * YT / 32]) return;
   const int64_t s = (int64_t)blockIdx.x * KC_THREADS + threadIdx.x;
   const int64_t y0 = (int64_t)blockIdx.y * YT;
@@ -117,16 +119,37 @@ __global__ void __launch_bounds__(KC_THREADS) kc_kernel(const __grid_constant__ 
   }
 }
 
+// A launch that may start under the end of the one before it in the stream (programmatic
+// dependent launch); the kernel waits for that one itself (griddepcontrol.wait).
+template <class... P, class... Q>
+void launch_under(void (*fn)(P...), dim3 grid, int threads, int smem, cudaStream_t st, const Q&... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = (size_t)smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, fn, static_cast<P>(args)...);
+}
+
 // one y-tile width per launch: 4, 8, 16 or 32 columns of C per thread
 template <int D, int AR, bool SUM>
 cudaError_t launch_kc_impl(const KParams& kp, const double* W, int64_t Y, int64_t ldw, double* C, int64_t ldc,
                            cudaStream_t st, const unsigned char* flag = nullptr) {
   const int yt = Y <= 4 ? 4 : (Y <= 8 ? 8 : (Y <= 16 || D == 4 ? 16 : 32));
   const dim3 grid((unsigned)((kp.S + KC_THREADS - 1) / KC_THREADS), (unsigned)((Y + yt - 1) / yt));
-  if (yt == 4) kc_kernel<D, AR, 4, SUM><<<grid, KC_THREADS, 0, st>>>(kp, W, Y, ldw, C, ldc, flag);
-  else if (yt == 8) kc_kernel<D, AR, 8, SUM><<<grid, KC_THREADS, 0, st>>>(kp, W, Y, ldw, C, ldc, flag);
-  else if (yt == 16) kc_kernel<D, AR, 16, SUM><<<grid, KC_THREADS, 0, st>>>(kp, W, Y, ldw, C, ldc, flag);
-  else if constexpr (D < 4) kc_kernel<D, AR, 32, SUM><<<grid, KC_THREADS, 0, st>>>(kp, W, Y, ldw, C, ldc, flag);
+  const auto go = [&](auto fn) {
+    if (flag) launch_under(fn, grid, KC_THREADS, 0, st, kp, W, Y, ldw, C, ldc, flag);
+    else fn<<<grid, KC_THREADS, 0, st>>>(kp, W, Y, ldw, C, ldc, flag);
+  };
+  if (yt == 4) go(kc_kernel<D, AR, 4, SUM>);
+  else if (yt == 8) go(kc_kernel<D, AR, 8, SUM>);
+  else if (yt == 16) go(kc_kernel<D, AR, 16, SUM>);
+  else if constexpr (D < 4) go(kc_kernel<D, AR, 32, SUM>);
   return cudaGetLastError();
 }
 

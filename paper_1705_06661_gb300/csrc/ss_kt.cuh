@@ -375,6 +375,7 @@ __global__ void __launch_bounds__(256) kt_prep_kernel(const __grid_constant__ KP
   __shared__ int left;
   __shared__ unsigned votes;
   const int tid = threadIdx.x, ch = blockIdx.x, yt = blockIdx.y;
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // kt_kernel, which waits for this grid
   const int nunit = ka.upre[npatterns(D)];
   if (tid < KT_COLS) colmax[tid] = collog[tid] = colzero[tid] = 0;
   if (tid < KT_CHUNK) {
@@ -550,6 +551,7 @@ __global__ void __launch_bounds__(KT_THREADS, 1) kt_kernel(const __grid_constant
   extern __shared__ __align__(128) unsigned char kt_smem[];
   __shared__ KtShared sh;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  asm volatile("griddepcontrol.wait;" ::: "memory");  // launched under the end of kt_prep_kernel
   if (ka.ytiles <= KT_VOTE && kt_all_left(ka, reinterpret_cast<unsigned*>(kt_smem))) return;
   if (tid == 0) {
     for (int i = 0; i < 3; i++) {
@@ -827,6 +829,7 @@ __global__ void __launch_bounds__(KT_THREADS, 1) kt_kernel(const __grid_constant
       }
   }
   if (!ok) report_timeout(kp);
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // KC, which waits for this grid
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -977,7 +980,7 @@ bool launch_kt(const KParams& kp, const double* W, int64_t Y, int64_t ldw, doubl
     kt_prep_kernel<D><<<dim3((unsigned)ka.nchunk, (unsigned)ka.ytiles), 256, 0, st>>>(kp, ka);
     *e = cudaGetLastError();
     if (*e == cudaSuccess) {
-      kt_kernel<D><<<(unsigned)grid, KT_THREADS, 2 * KT_STAGE, st>>>(kp, ka);
+      launch_under(kt_kernel<D>, dim3((unsigned)grid), KT_THREADS, 2 * KT_STAGE, st, kp, ka);
       *e = cudaGetLastError();
     }
     if (*e == cudaSuccess) *e = launch_kc_impl<D, AR_EXACT, true>(kp, ka.W, ka.Y, ldw, ka.C, ldc, st, ka.flag);
