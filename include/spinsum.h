@@ -200,7 +200,8 @@ int spinsum_4d_host(int dtype, const int64_t ext[8], const void* A, const int64_
  * bytes per tuple and 32 columns; where those exceed 128 MB, columns are taken
  * in slabs as far as the positions allow, and none takes more than 2 GB) from a
  * pool of the library that keeps at most 128 MB between calls; where none can be had the FP64 path runs.
- * Under stream capture the FP64 path runs too: the graph holds no allocation.
+ * Under stream capture the workspace belongs to the graph (a user object; no
+ * allocation nodes) and goes back to the pool behind a later call on the device.
  * Errors: SPINSUM_ERR_ARG (bad d, extents,
  * leading dimensions, pointers or mode bits), SPINSUM_ERR_ALIAS (C overlaps A
  * or W), SPINSUM_ERR_CUDA. Asynchronous on `stream`.

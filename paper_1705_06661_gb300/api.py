@@ -124,8 +124,8 @@ def contract(A: torch.Tensor, coef, W: torch.Tensor, *, d: int | None = None, ou
 
     Calls of more than 256 spectator positions with integer coefficients run on
     the tensor cores, S(A) and W as integers on one scale per row (column) and
-    192 tuples; where magnitudes are too far apart for that, under stream
-    capture and with strict=True they run in FP64. The bits of the result
+    192 tuples; where magnitudes are too far apart for that and with strict=True
+    they run in FP64. The bits of the result
     depend on that choice (and so does their equality with the unfused pair of
     calls); strict=True makes it, and takes no workspace."""
     if d is None:

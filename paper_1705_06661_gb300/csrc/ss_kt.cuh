@@ -54,6 +54,8 @@
 #include "ss_tma.cuh"
 
 #include <algorithm>
+#include <atomic>
+#include <new>
 
 #include <cuda_fp16.h>
 
@@ -870,6 +872,73 @@ inline cudaMemPool_t kt_pool(int dev) {
   return (cudaMemPool_t)(uintptr_t)v;
 }
 
+// Workspaces of captured calls. Allocation nodes would keep a graph from being
+// instantiated twice or put into another, and KC, which needs none, takes up to twelve
+// times as long; so the graph holds a workspace from the pool as a user object, and a later
+// call gives it back (no CUDA call may be made where the graph's end is reported).
+struct KtHeld {
+  void* ws;
+  int dev;
+  KtHeld* next;
+};
+inline std::atomic<KtHeld*>& kt_dead() {
+  static std::atomic<KtHeld*> head{nullptr};
+  return head;
+}
+inline void CUDART_CB kt_retire(void* held) {
+  KtHeld* h = static_cast<KtHeld*>(held);
+  h->next = kt_dead().load(std::memory_order_relaxed);
+  while (!kt_dead().compare_exchange_weak(h->next, h, std::memory_order_release, std::memory_order_relaxed)) {
+  }
+}
+// the workspaces of device dev whose graphs are gone, back to the pool in st's order
+inline void kt_reap(int dev, cudaStream_t st) {
+  if (kt_dead().load(std::memory_order_relaxed) == nullptr) return;
+  for (KtHeld* h = kt_dead().exchange(nullptr, std::memory_order_acquire); h != nullptr;) {
+    KtHeld* const next = h->next;
+    if (h->dev != dev) {
+      kt_retire(h);
+    } else {
+      if (cudaFreeAsync(h->ws, st) != cudaSuccess) cudaGetLastError();
+      delete h;
+    }
+    h = next;
+  }
+}
+inline bool kt_graph_workspace(cudaMemPool_t pool, int dev, cudaGraph_t graph, size_t bytes, unsigned char** ws) {
+  // the allocation goes to a stream of its own, outside the capture
+  static DeviceCache cache;
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  if (cudaThreadExchangeStreamCaptureMode(&mode) != cudaSuccess) return false;
+  long long v = 0;
+  const int rc = cache.get(dev, &v, [](long long* val) {
+    cudaStream_t s = nullptr;
+    const cudaError_t err = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking);
+    *val = (long long)(uintptr_t)s;
+    return (int)err;
+  });
+  const cudaStream_t own = (cudaStream_t)(uintptr_t)v;
+  KtHeld* const held = new (std::nothrow) KtHeld{nullptr, dev, nullptr};
+  bool ok = rc == 0 && held != nullptr && cudaMallocFromPoolAsync((void**)ws, bytes, pool, own) == cudaSuccess;
+  if (ok) {
+    held->ws = *ws;
+    cudaUserObject_t obj = nullptr;
+    ok = cudaStreamSynchronize(own) == cudaSuccess &&
+         cudaUserObjectCreate(&obj, held, kt_retire, 1, cudaUserObjectNoDestructorSync) == cudaSuccess;
+    if (!ok) {
+      cudaFreeAsync(*ws, own);
+      delete held;
+    } else if (cudaGraphRetainUserObject(graph, obj, 1, cudaGraphUserObjectMove) != cudaSuccess) {
+      cudaUserObjectRelease(obj, 1);  // kt_retire: given back by a later call
+      ok = false;
+    }
+  } else {
+    delete held;
+  }
+  cudaThreadExchangeStreamCaptureMode(&mode);
+  return ok;
+}
+
 // Whether KT takes the contraction: exact arithmetic with integer coefficients
 // (the operator's 1-norm is then at most 127, so the limb sums stay below 2^31),
 // more than two row tiles (smaller calls stay with KC, whose FP64 sums equal those of
@@ -917,10 +986,9 @@ bool launch_kt(const KParams& kp, const double* W, int64_t Y, int64_t ldw, doubl
   ka.nchunk = (int)((units + KT_UPC - 1) / KT_UPC);
   const int64_t ct = Y <= 4 ? 4 : (Y <= 8 ? 8 : (Y <= 16 || D == 4 ? 16 : 32)), kc_cols = (Y + ct - 1) / ct * ct;
   if (2.7 * KT_CHUNK * ka.nchunk * ka.ytiles > (double)T * kc_cols || (double)kp.S * T * kc_cols < 1e6) return false;
-  // A call under capture takes KC, which needs no workspace: one in the graph's own
-  // allocation nodes would keep the graph from being instantiated twice or put into another.
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+  cudaGraph_t graph = nullptr;  // that the call is captured into
+  if (cudaStreamGetCaptureInfo(st, &cap, nullptr, &graph) != cudaSuccess || cap == cudaStreamCaptureStatusInvalidated) {
     cudaGetLastError();
     return false;
   }
@@ -957,11 +1025,14 @@ bool launch_kt(const KParams& kp, const double* W, int64_t Y, int64_t ldw, doubl
   const int64_t nd = slab * ka.nchunk, bw = nd * 4 * KT_WST, be = nd * KT_COLS * 4, br = nd * 8;
   unsigned char* ws = nullptr;
   cudaMemPool_t pool = kt_pool(dev);
+  const size_t bytes = (size_t)(bw + be + br + bt + bp + slab * rows);
   if (!pool || bw > (2LL << 30) ||
-      cudaMallocFromPoolAsync((void**)&ws, (size_t)(bw + be + br + bt + bp + slab * rows), pool, st) != cudaSuccess) {
+      (graph ? !kt_graph_workspace(pool, dev, graph, bytes, &ws)
+             : cudaMallocFromPoolAsync((void**)&ws, bytes, pool, st) != cudaSuccess)) {
     cudaGetLastError();
     return false;  // KC needs no workspace
   }
+  if (!graph) kt_reap(dev, st);
   ka.wdig = ws;
   ka.wexp = reinterpret_cast<unsigned*>(ws + bw);
   ka.room = reinterpret_cast<int*>(ws + bw + be);
@@ -986,8 +1057,10 @@ bool launch_kt(const KParams& kp, const double* W, int64_t Y, int64_t ldw, doubl
     if (*e == cudaSuccess) *e = launch_kc_impl<D, AR_EXACT, true>(kp, ka.W, ka.Y, ldw, ka.C, ldc, st, ka.flag);
   }
   count_launches((int)(3 * nslab - 1));
-  const cudaError_t f = cudaFreeAsync(ws, st);
-  if (*e == cudaSuccess) *e = f;
+  if (!graph) {
+    const cudaError_t f = cudaFreeAsync(ws, st);
+    if (*e == cudaSuccess) *e = f;
+  }
   return true;
 }
 

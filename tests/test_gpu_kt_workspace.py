@@ -114,3 +114,30 @@ def test_launches_are_counted():
         ss.contract(a, coef, w, factorized=True, strict=strict)
         assert ss.spinsum_launch_count(reset=True) == n
     torch.cuda.synchronize()
+
+
+def test_captured_calls_keep_the_bits_and_give_the_workspace_back():
+    """A replay gives the bits of the eager call, on new inputs too; the workspaces of destroyed graphs go
+    back to the pool, whose size stays that of a few of them."""
+    import torch
+    import paper_1705_06661_gb300 as ss
+    d, O, S, Y = 3, 30, 300, 64                            # 24 MB of digits
+    coef = wl.table2(1)
+    A = [_place(wl.uniform(7 + k, (S, 1, 1) + (O,) * d)) for k in range(2)]
+    w = _place(wl.uniform(9, (Y, O ** d)))
+    a, out = ss.colmajor_like(A[0]), ss.colmajor_empty((S, 1, 1, Y))
+    want = [ss.contract(x, coef, w, factorized=True) for x in A]
+    torch.cuda.synchronize()
+    free0 = torch.cuda.mem_get_info()[0]
+    for k in range(16):
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g):
+            ss.contract(a, coef, w, out=out, factorized=True)
+        a.copy_(A[k % 2])
+        g.replay()
+        assert torch.equal(out, want[k % 2])
+        g.replay()
+        del g
+        assert torch.equal(ss.contract(A[1], coef, w, factorized=True), want[1])
+    torch.cuda.synchronize()
+    assert free0 - torch.cuda.mem_get_info()[0] <= 160 << 20
