@@ -522,10 +522,12 @@ int plan_one(const Request& r, Launch* L) {
       // of its tuple: about as long as SETUP chunks) and its chunks; all blocks share the
       // resident CTAs, and the last ones run out on their own. us per call with 1, 2, 4, .. chunks
       // per block: A[8000,10^3] FP64 32.8, 30.6, 28.6, 44 (16); A[64000,6^3] 46.5 (3), 43.7 (4),
-      // 55 (16); A[4096,6^4] 31 (2), 28.6 (4), 37 (8), 66 (16); A[1000,10^4] 58 (1), 41.7 (4).
+      // 55 (16); A[4096,6^4] 31 (2), 28.6 (4), 37 (8), 66 (16); A[1000,10^4] 58 (1), 41.7 (4). (A
+      // set-up of 1.5 chunks for d <= 3: as good on single calls, 32 chained blocks 3014 us
+      // against 2967.)
       int64_t orbits = 0;
       for (int p = 0; p < np; p++) orbits += kp.norb[p];
-      const double setup = d == 4 ? 3.0 : 1.5, resident = 152.0 * (d == 4 ? 3 : 4);
+      const double setup = d == 4 ? 3.0 : 2.5, resident = 152.0 * (d == 4 ? 3 : 4);
       double least = 1e300;
       int64_t best = cpb0;
       for (int64_t c = cpb0; c >= 1; c--) {
